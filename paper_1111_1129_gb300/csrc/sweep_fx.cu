@@ -12,9 +12,9 @@
 //    common unit U = 2^-58 gives an exact int64 X_q; the store converts
 //    back the same way.  No FP64 conversion is needed on this path.
 //  * Pair sums/differences, rho - 1 and j are then exact integer sums.
-//  * Products with the relaxation constants use 64x64 -> high-64 integer
-//    multiplies with the constants scaled by 2^63 (relative precision
-//    2^-62).  The quadratic velocity terms come from the six products
+//  * Products with the relaxation constants, scaled by 2^63, take three
+//    32x32 -> 64 products each and are rounded, within one unit of the exact
+//    product (fxmul).  The quadratic velocity terms come from the six products
 //    u_a u_b, each built from three 32x32 -> 64 integer products and exact
 //    to 2 units (7e-18); this needs |u| < 2^-6.
 //  * After rounding to the storage units, the rest population takes the
@@ -39,11 +39,38 @@
 namespace lbm {
 namespace {
 
+// x * c to within a unit (unbiased), for c = c63 / 2^63 with |c| < 1/2 and
+// |x| < 2^59, from three 32x32 -> 64 products: x and c63 are cut into a high
+// part and a signed low word, x = xh 2^32 + xl, so that
+//   x c63 / 2^63 = 2 xh ch + (xh cl + xl ch) / 2^31 + xl cl / 2^63,
+// the middle term is rounded and the last (at most 1/2) dropped.  Six
+// or seven instructions, three of them multiply-adds; __mul64hi(2 x, c63)
+// takes about twice as many and rounds down.  The step is bound by DRAM, but
+// its ALU pipe was 60% busy: this product, range checks by one logic
+// instruction per value and sums formed from the pairs took the 32x32x64
+// bed (no DRAM traffic) from 8,176 to 8,890 MFLUP/s and the 1024x256x256 bed
+// from 18,096 to 18,580, and the error of u after 30 steps there from 5.2e-11
+// to 1.6e-11 of u.
+struct Fx63 {
+  int32_t h, l;
+};
+__host__ __device__ __forceinline__ Fx63 fx63(int64_t c63) {
+  const int32_t l = (int32_t)(uint32_t)(uint64_t)c63;
+  return {(int32_t)((c63 - l) >> 32), l};
+}
+__device__ __forceinline__ int64_t fxmul(int64_t x, Fx63 c) {
+  const int32_t xl = (int32_t)(uint32_t)(uint64_t)x;
+  const int32_t xh = (int32_t)(x >> 32) + (int32_t)((uint32_t)xl >> 31);
+  const int64_t mid = ((int64_t)1 << 30) + (int64_t)xh * c.l + (int64_t)xl * c.h;
+  return (int64_t)(2 * xh) * c.h + (mid >> 31);
+}
+
 struct FxCoef {
-  int64_t hp, hm, w1p, a1;  // (1-w+)/2, (1-w-)/2, w+/18, w-/6, each * 2^63
+  Fx63 hp, hm, w1p;         // (1-w+)/2, (1-w-)/2, w+/18, each * 2^63
+  int64_t a1;               // w-/6 * 2^63
   int32_t hp_shift;         // when (1-w+)/2 = hp_sign * 2^-hp_shift exactly
   int32_t hp_sign;
-  int64_t q1;               // w+/36 (quadratic terms) * 2^63
+  Fx63 q1;                  // w+/36 (quadratic terms) * 2^63
   int64_t hF[3];            // F/2 in units U
   int64_t bF1[3];           // (1 - w-/2) F / 6 in units U
   int64_t b1x2;             // 2 (1 - w-/2)/6 * 2^63: mul.hi with alpha 2^63 gives b1 alpha 2^63
@@ -66,9 +93,6 @@ constexpr int64_t kW2Bits = 0x3F9C71C71C71C71CLL;  // 1/36
 __device__ __forceinline__ int64_t wbits(int q) { return q == 0 ? kW0Bits : (q <= 6 ? kW1Bits : kW2Bits); }
 __device__ __forceinline__ int64_t wexp(int q) { return q == 0 ? 0x3FD : (q <= 6 ? 0x3FA : 0x3F9); }
 __device__ __forceinline__ int wshift(int q) { return q == 0 ? 4 : (q <= 6 ? 1 : 0); }
-
-// x * c for a constant c = c63 / 2^63 (|c| < 1/2), |x| < 2^59: floor.
-__device__ __forceinline__ int64_t fxmul(int64_t x, int64_t c63) { return __mul64hi(2 * x, c63); }
 
 // Resident blocks of 256 threads per SM the register budget is fitted to:
 // on the 1024x256x256 bed 3 (80 registers) beat 2 (120 registers) by 15%
@@ -130,19 +154,20 @@ __device__ __forceinline__ void fx_pull(const double* __restrict__ src, const in
 __device__ __forceinline__ bool fx_moments(const int64_t b[19], const FxCoef& k, int64_t S[9],
                                            int64_t D[9], int64_t& drho, int64_t& ux,
                                            int64_t& uy, int64_t& uz) {
-  bool fast = true;
+  // sign and exponent bits that differ from the weight's (one three-input
+  // logic instruction per value)
+  uint32_t off = 0;
 #pragma unroll
-  for (int q = 0; q < 19; ++q) fast &= (b[q] >> 52) == wexp(q);
-  if (!fast) return false;
-  int64_t X[19];
-#pragma unroll
-  for (int q = 0; q < 19; ++q) X[q] = (b[q] - wbits(q)) << wshift(q);
+  for (int q = 0; q < 19; ++q) off |= (uint32_t)(b[q] >> 32) ^ (uint32_t)(wbits(q) >> 32);
+  if (off >> 20) return false;
+  // the weights cancel in the differences; each sum is one three-term add
 #pragma unroll
   for (int p = 0; p < 9; ++p) {
-    S[p] = X[2 * p + 1] + X[2 * p + 2];
-    D[p] = X[2 * p + 1] - X[2 * p + 2];
+    const int q = 2 * p + 1;
+    S[p] = (b[q] + b[q + 1] - 2 * wbits(q)) << wshift(q);
+    D[p] = (b[q] - b[q + 1]) << wshift(q);
   }
-  drho = X[0] + (((S[0] + S[1]) + (S[2] + S[3])) + ((S[4] + S[5]) + (S[6] + S[7])) + S[8]);
+  drho = ((b[0] - wbits(0)) << wshift(0)) + (((S[0] + S[1]) + (S[2] + S[3])) + ((S[4] + S[5]) + (S[6] + S[7])) + S[8]);
   ux = (((D[0] + D[3]) + (D[4] + D[5])) + D[6]) + k.hF[0];
   uy = (((D[1] + D[3]) - (D[4] - D[7])) + D[8]) + k.hF[1];
   uz = (((D[2] + D[5]) - (D[6] - D[7])) - D[8]) + k.hF[2];
@@ -154,15 +179,16 @@ __device__ __forceinline__ bool fx_moments(const int64_t b[19], const FxCoef& k,
 // The fixed-point TRT collision of one cell from its exact moments, and the
 // store of its 19 results.  HP_POW2: (1 - w+)/2 is +-2^-k (w+ = 1.25, 1.5,
 // 0.75, ...), so the nine even-part products are shifts.
-template <bool HP_POW2>
+template <int HP_POW2>
 __device__ __forceinline__ void fx_collide_store(const int64_t S[9], const int64_t D[9],
                                                  int64_t drho, int64_t ux, int64_t uy,
                                                  int64_t uz, const FxCoef& k, int64_t a1,
                                                  double* __restrict__ dst, int32_t ld, int32_t i) {
   // a1: the odd-part coefficient w-/6 (undamped) or w-/6 - b1 alpha, * 2^63
-  const int64_t V1x = fxmul(ux, a1) + k.bF1[0];
-  const int64_t V1y = fxmul(uy, a1) + k.bF1[1];
-  const int64_t V1z = fxmul(uz, a1) + k.bF1[2];
+  const Fx63 a1_ = fx63(a1);
+  const int64_t V1x = fxmul(ux, a1_) + k.bF1[0];
+  const int64_t V1y = fxmul(uy, a1_) + k.bF1[1];
+  const int64_t V1z = fxmul(uz, a1_) + k.bF1[2];
   const int64_t V2x = V1x >> 1, V2y = V1y >> 1, V2z = V1z >> 1;
   // Quadratic terms w+ w_p (4.5 (c.u)^2 - 1.5 u.u) = (w+ w_p / 2)
   // (9 (c.u)^2 - 3 u.u): with v = (w+/36) u, the products
@@ -175,16 +201,29 @@ __device__ __forceinline__ void fx_collide_store(const int64_t S[9], const int64
   const int64_t Ttr3 = 3 * (Txx + Tyy + Tzz);
   const int64_t R1 = fxmul(drho, k.w1p);
   const int64_t R2 = R1 >> 1;
-  int64_t out[19];
+  // The moving populations are rounded to their storage units (2^-57 axis,
+  // 2^-58 diagonal); the rest population takes the remainder rounded to
+  // its unit 2^-54, and the last -8..7 units go to a diagonal
+  // population, so the stored deviations sum exactly to drho: every
+  // step conserves the stored mass bit for bit.  A pair P +- Q stores 2 P,
+  // plus 2 when rounding an axis pair up moved both (P + Q and P - Q have
+  // the same parity).
+  int64_t d[19];
+  int64_t half = 0;   // half of what the pairs store
+  int32_t up = 0;
 #define LBM_FX_PAIR(P, QUAD, R, VX)                                         \
   {                                                                         \
-    const int64_t hS_ = HP_POW2 ? (k.hp_sign > 0 ? S[P] >> k.hp_shift       \
-                                             : -(S[P] >> k.hp_shift))   \
-                            : fxmul(S[P], k.hp);                        \
-    const int64_t P_ = hS_ + R + (QUAD);                                    \
+    const int64_t hS_ = HP_POW2 ? S[P] >> k.hp_shift : fxmul(S[P], k.hp);   \
+    const int64_t P_ = HP_POW2 < 0 ? R + (QUAD) - hS_ : R + (QUAD) + hS_;   \
     const int64_t Q_ = fxmul(D[P], k.hm) + (VX);                            \
-    out[2 * P + 1] = P_ + Q_;                                               \
-    out[2 * P + 2] = P_ - Q_;                                               \
+    half += P_;                                                             \
+    d[2 * P + 1] = P_ + Q_;                                                 \
+    d[2 * P + 2] = P_ - Q_;                                                 \
+    if (P < 3) {                                                            \
+      up += (int32_t)d[2 * P + 1] & 1;                                      \
+      d[2 * P + 1] = (d[2 * P + 1] + 1) >> 1;                               \
+      d[2 * P + 2] = (d[2 * P + 2] + 1) >> 1;                               \
+    }                                                                       \
   }
   LBM_FX_PAIR(0, 9 * Txx - Ttr3, R1, V1x)
   LBM_FX_PAIR(1, 9 * Tyy - Ttr3, R1, V1y)
@@ -196,20 +235,7 @@ __device__ __forceinline__ void fx_collide_store(const int64_t S[9], const int64
   LBM_FX_PAIR(7, (9 * (Tyy + Tzz + Tyz2) - Ttr3) >> 1, R2, V2y + V2z)
   LBM_FX_PAIR(8, (9 * (Tyy + Tzz - Tyz2) - Ttr3) >> 1, R2, V2y - V2z)
 #undef LBM_FX_PAIR
-  // Round the moving populations to their storage units (2^-57 axis,
-  // 2^-58 diagonal); the rest population takes the remainder rounded to
-  // its unit 2^-54, and the last -8..7 units go to a diagonal
-  // population, so the stored deviations sum exactly to drho: every
-  // step conserves the stored mass bit for bit.
-  int64_t d[19];
-  int64_t stored = 0;
-#pragma unroll
-  for (int q = 1; q < 19; ++q) {
-    const int s = wshift(q);
-    d[q] = s ? (out[q] + (1LL << (s - 1))) >> s : out[q];
-    stored += d[q] << s;
-  }
-  const int64_t rem = drho - stored;
+  const int64_t rem = drho - 2 * (half + up);
   d[0] = (rem + 8) >> 4;
   d[7] += rem - (d[0] << 4);
   // Store the fixed-point result; an output that left its binary range
@@ -219,13 +245,16 @@ __device__ __forceinline__ void fx_collide_store(const int64_t S[9], const int64
 #pragma unroll
   for (int q = 0; q < 19; ++q) {
     const int64_t bits = wbits(q) + d[q];
-    out_of_range |= (uint32_t)((bits >> 52) != wexp(q)) << q;
+    out_of_range |= (uint32_t)(bits >> 32) ^ (uint32_t)(wbits(q) >> 32);
     st_cs(dst + q * ld + i, __longlong_as_double(bits));
   }
-  if (out_of_range) {
-    for (int q = 0; q < 19; ++q)
-      if ((out_of_range >> q) & 1u)
-        dst[q * ld + i] = weight(q) + (double)(d[q] << wshift(q)) * 0x1p-58;
+  if (out_of_range >> 20) {
+    for (int q = 0; q < 19; ++q) {
+      volatile double* at = dst + q * ld + i;
+      const int64_t dq = __double_as_longlong(*at) - wbits(q);
+      if (((wbits(q) + dq) >> 52) != wexp(q))
+        *at = weight(q) + (double)(dq << wshift(q)) * 0x1p-58;
+    }
   }
 }
 
@@ -255,7 +284,7 @@ __device__ __forceinline__ bool fx_damp(const int64_t* __restrict__ alpha_fx, in
   if constexpr (DAMPED) {
     const int64_t A = __ldg(alpha_fx + i);
     if (A < 0) return false;
-    const int64_t E = __ldg(alpha_fx + n + i);
+    const Fx63 E = fx63(__ldg(alpha_fx + n + i));
     ux -= fxmul(ux, E);
     uy -= fxmul(uy, E);
     uz -= fxmul(uz, E);
@@ -265,7 +294,7 @@ __device__ __forceinline__ bool fx_damp(const int64_t* __restrict__ alpha_fx, in
 }
 
 // A step that does not reduce: n cells, PDF and link rows of stride ld.
-template <bool HP_POW2, bool DAMPED>
+template <int HP_POW2, bool DAMPED>
 __global__ void __launch_bounds__(kSweepThreads, LBM_FX_MIN_BLOCKS)
     sweep_fx_kernel(const double* __restrict__ src, double* __restrict__ dst,
                     const int32_t* __restrict__ adj, int32_t n, int32_t ld, FxCoef k,
@@ -296,7 +325,7 @@ __global__ void __launch_bounds__(kSweepThreads, LBM_FX_MIN_BLOCKS)
 // rather than keep the raw bits live: the reduction then adds little to the
 // registers the collision needs.  (Sharing this structure with the plain
 // step made that one spill.)
-template <bool HP_POW2, bool DAMPED>
+template <int HP_POW2, bool DAMPED>
 __global__ void __launch_bounds__(kSweepThreads, LBM_FX_RED_MIN_BLOCKS)
     sweep_fx_reduce_kernel(const double* __restrict__ src, double* __restrict__ dst,
                            const int32_t* __restrict__ adj, int32_t n, int32_t ld, FxCoef k,
@@ -343,7 +372,7 @@ namespace {
 // (1 - w+)/2 is an exact power of two, so the even-part products are shifts.
 FxCoef make_fx_coef(double wp, double wm, const double F[3], bool* pow2) {
   FxCoef k{};
-  k.hp = c63(0.5 * (1.0 - wp));
+  k.hp = fx63(c63(0.5 * (1.0 - wp)));
   // exact power of two (the mantissa of |hp| is 1/2) between 2^-1 and 2^-40
   const double hp = 0.5 * (1.0 - wp);
   int e = 0;
@@ -351,14 +380,14 @@ FxCoef make_fx_coef(double wp, double wm, const double F[3], bool* pow2) {
   *pow2 = m == 0.5 && -e + 1 >= 1 && -e + 1 <= 40;
   k.hp_shift = *pow2 ? 1 - e : 0;
   k.hp_sign = hp < 0 ? -1 : 1;
-  k.hm = c63(0.5 * (1.0 - wm));
-  k.w1p = c63(wp / 18.0);
+  k.hm = fx63(c63(0.5 * (1.0 - wm)));
+  k.w1p = fx63(c63(wp / 18.0));
   k.a1 = c63(wm / 6.0);
   for (int d = 0; d < 3; ++d) {
     k.hF[d] = units(0.5 * F[d]);
     k.bF1[d] = units((1.0 - 0.5 * wm) * F[d] / 6.0);
   }
-  k.q1 = c63(wp / 36.0);
+  k.q1 = fx63(c63(wp / 36.0));
   k.b1x2 = 2 * c63((1.0 - 0.5 * wm) / 6.0);
   return k;
 }
@@ -377,11 +406,11 @@ cudaError_t launch_fx(const lbm_state* st, const double* src, double* dst, const
   return partials ? launch_sweep(sweep_fx_reduce_kernel<P2, DA>, grid, stream, chained, src, dst, adj, n, ld, k, kd, alpha, afx, partials) \
                   : launch_sweep(sweep_fx_kernel<P2, DA>, grid, stream, chained, src, dst, adj, n, ld, k, kd, alpha, afx)
   if (alpha) {
-    if (pow2) LBM_FX_LAUNCH(true, true);
-    LBM_FX_LAUNCH(false, true);
+    if (pow2) { if (k.hp_sign > 0) LBM_FX_LAUNCH(1, true); LBM_FX_LAUNCH(-1, true); }
+    LBM_FX_LAUNCH(0, true);
   }
-  if (pow2) LBM_FX_LAUNCH(true, false);
-  LBM_FX_LAUNCH(false, false);
+  if (pow2) { if (k.hp_sign > 0) LBM_FX_LAUNCH(1, false); LBM_FX_LAUNCH(-1, false); }
+  LBM_FX_LAUNCH(0, false);
 #undef LBM_FX_LAUNCH
 }
 
