@@ -136,12 +136,13 @@ int lbm_ordering_keys(const int32_t dims[3], lbm_ordering ord, uint64_t* keys_de
  *            fluid cells ranked by key), inv[nx*ny*nz] (n, or -1 for solid)
  *            and the adjacency.  The states keep their arrays in rows of
  *            L slots, L = N rounded up to 64, so that every row starts on a
- *            128-byte boundary; the adjacency is stored in that layout
- *            (18 rows of L, entries r*L + m; 72 bytes per L), which the
- *            steps read.  When L = N that is adj[18*N] of the layout above;
- *            otherwise adj[18*N] is derived from it on its first request
- *            (lbm_sparse_info, lbm_adjoint_create, lbm_state_create_batched)
- *            and then kept.
+ *            128-byte boundary; the adjacency the steps read names slots
+ *            r*L + m, as int32 (18 rows of L, 72 bytes per L) or, for larger lists
+ *            (more than 311,296 cells on GB300), in 16 bits per link and a table of neighbourhoods per 64 cells (38
+ *            bytes per L).  adj[18*N] of the layout above is derived from it
+ *            on its first request (lbm_sparse_info, lbm_adjoint_create,
+ *            lbm_state_create_batched) and then kept; with int32 links and
+ *            L = N it is the same array.
  * The call synchronises `stream` (to learn N, and again before returning,
  * so the flags may be released afterwards).  Errors: LBM_EINVAL,
  * LBM_EFLAGS, LBM_EOVERFLOW (19*L >= 2^31), LBM_ENOMEM, LBM_ECUDA.
@@ -152,7 +153,7 @@ int lbm_build_sparse(const uint8_t* flags, const int32_t dims[3], lbm_ordering o
 /*
  * Read-only views of a sparse representation.  Any out pointer may be NULL.
  * The device pointers stay owned by the handle.  adj_dev is adj[18*N] of the
- * layout above; when N is not a multiple of 64 the first request builds it
+ * layout above; unless the steps' links are that array the first request builds it
  * (72 bytes per cell of device memory, one kernel on the handle's stream,
  * which the call then synchronises) and may fail with LBM_ENOMEM.
  */

@@ -679,8 +679,8 @@ struct Runner {
       chained = true;
       return;
     }
-    if (alpha) launch(sweep_kernel<PREC, true, kNoReduce>, src, dst, st->sp->adj, n, n, k, alpha, (double*)nullptr);
-    else launch(sweep_kernel<PREC, false, kNoReduce>, src, dst, st->sp->adj, n, n, k, alpha, (double*)nullptr);
+    if (alpha) launch(sweep_kernel<PREC, true, kNoReduce>, src, dst, Links{st->sp->adj, nullptr, nullptr}, n, n, k, alpha, (double*)nullptr);
+    else launch(sweep_kernel<PREC, false, kNoReduce>, src, dst, Links{st->sp->adj, nullptr, nullptr}, n, n, k, alpha, (double*)nullptr);
   }
   void seed(const S* f_prev) const {
     if constexpr (PREC == LBM_F64X) {

@@ -220,6 +220,25 @@ __global__ void __launch_bounds__(kTileThreads)
   }
 }
 
+// Fluid index of the upwind neighbour of box cell (x, y, z) in direction q, or
+// -1: the link bounces back (Sec. 2).
+__device__ __forceinline__ int32_t upwind(int q, int32_t x, int32_t y, int32_t z, int32_t nx,
+                                          int32_t ny, int32_t nz, uint32_t periodic,
+                                          const int32_t* __restrict__ inv) {
+  int32_t sx = x - cx(q), sy = y - cy(q), sz = z - cz(q);
+  bool inside = true;
+  if (sx < 0 || sx >= nx) {
+    if (periodic & 1u) sx = sx < 0 ? sx + nx : sx - nx; else inside = false;
+  }
+  if (sy < 0 || sy >= ny) {
+    if (periodic & 2u) sy = sy < 0 ? sy + ny : sy - ny; else inside = false;
+  }
+  if (sz < 0 || sz >= nz) {
+    if (periodic & 4u) sz = sz < 0 ? sz + nz : sz - nz; else inside = false;
+  }
+  return inside ? inv[sx + nx * (sy + ny * sz)] : -1;
+}
+
 // Pull adjacency (Sec. 2): source slot of direction i for fluid cell n, in
 // rows of ld >= n entries naming slot r ld + m (ld = n: the public layout).
 __global__ void adjacency_kernel(int32_t nx, int32_t ny, int32_t nz, uint32_t periodic,
@@ -232,36 +251,92 @@ __global__ void adjacency_kernel(int32_t nx, int32_t ny, int32_t nz, uint32_t pe
   const int32_t x = c % nx, y = (c / nx) % ny, z = c / (nx * ny);
 #pragma unroll
   for (int q = 1; q < 19; ++q) {
-    int32_t sx = x - cx(q), sy = y - cy(q), sz = z - cz(q);
-    bool inside = true;
-    if (sx < 0 || sx >= nx) {
-      if (periodic & 1u) sx = sx < 0 ? sx + nx : sx - nx; else inside = false;
-    }
-    if (sy < 0 || sy >= ny) {
-      if (periodic & 2u) sy = sy < 0 ? sy + ny : sy - ny; else inside = false;
-    }
-    if (sz < 0 || sz >= nz) {
-      if (periodic & 4u) sz = sz < 0 ? sz + nz : sz - nz; else inside = false;
-    }
-    int32_t m = -1;
-    if (inside) m = inv[sx + nx * (sy + ny * sz)];
+    const int32_t m = upwind(q, x, y, z, nx, ny, nz, periodic, inv);
     adj[(q - 1) * ld + i] = m >= 0 ? q * ld + m : opp(q) * ld + i;
   }
 }
 
-// The public links (rows of n, slot q n + m) from links in rows of ld > n
+// ---- short links (lbm::Links) -------------------------------------------------
+// One warp per tile of kLinkTile cells, two cells per lane.  The tile's page
+// list grows in the order in which pages are met; lane e holds entry e.  A row
+// of 32 links mostly meets one or two pages.
+__global__ void __launch_bounds__(256)
+    short_links_kernel(int32_t nx, int32_t ny, int32_t nz, uint32_t periodic,
+                       const int32_t* __restrict__ cells, const int32_t* __restrict__ inv,
+                       int32_t n, int32_t ld, uint16_t* __restrict__ code,
+                       int32_t* __restrict__ pages, int32_t* overflow) {
+  const int32_t tile = (int32_t)(blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32);
+  if (tile >= ld / kLinkTile) return;
+  const int lane = threadIdx.x & 31;
+  int32_t mine = -1, count = 0;   // this lane's page, pages listed
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    const int32_t j = 32 * h + lane, i = tile * kLinkTile + j;
+    const int32_t c = i < n ? cells[i] : 0;
+    const int32_t x = c % nx, y = (c / nx) % ny, z = c / (nx * ny);
+    int32_t m[18];
+#pragma unroll
+    for (int q = 1; q < 19; ++q)
+      m[q - 1] = i < n ? upwind(q, x, y, z, nx, ny, nz, periodic, inv) : -1;
+#pragma unroll
+    for (int q = 1; q < 19; ++q) {
+      const int32_t page = m[q - 1] / kLinkPage;
+      uint32_t word = (uint32_t)((q & 1) ? kLinkPages : kLinkPages + 1) * kLinkPage + (uint32_t)j;
+      bool open = m[q - 1] >= 0;
+      for (uint32_t left; (left = __ballot_sync(0xffffffffu, open)) != 0;) {
+        const int32_t p = __shfl_sync(0xffffffffu, page, __ffs(left) - 1);
+        const uint32_t hit = __ballot_sync(0xffffffffu, mine == p);
+        const int e = hit ? __ffs(hit) - 1 : count++;
+        if (e >= kLinkPages) {   // too many pages: the caller takes 32-bit links
+          if (lane == 0) *overflow = 1;
+          return;
+        }
+        if (!hit && lane == e) mine = p;
+        if (open && page == p) {
+          word = (uint32_t)e * kLinkPage + (uint32_t)(m[q - 1] % kLinkPage);
+          open = false;
+        }
+      }
+      code[(q - 1) * ld + i] = (uint16_t)word;
+    }
+  }
+  const int32_t first = tile * kLinkTile;
+  pages[32 * tile + lane] = lane == kLinkPages       ? first + ld
+                            : lane == kLinkPages + 1 ? first - ld
+                                                     : (mine < 0 ? 0 : mine * kLinkPage);
+}
+
+// The public links (rows of n, slot q n + m) from links in rows of ld
 // (slot r ld + m); grid (cells, 18 rows).
-__global__ void public_links_kernel(const int32_t* __restrict__ adj_ld, int32_t ld, int32_t n,
+__global__ void public_links_kernel(Links links, int32_t ld, int32_t n,
                                     int32_t* __restrict__ adj) {
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int32_t q = (int32_t)blockIdx.y;
+  const int32_t r = (int32_t)blockIdx.y;
   if (i >= n) return;
-  const uint32_t s = (uint32_t)adj_ld[q * ld + i];
-  const uint32_t r = s / (uint32_t)ld;
-  adj[q * n + i] = (int32_t)(r * (uint32_t)n + (s - r * (uint32_t)ld));
+  if (links.wide) {
+    const uint32_t s = (uint32_t)links.wide[r * ld + i];
+    const uint32_t q = s / (uint32_t)ld;
+    adj[r * n + i] = (int32_t)(q * (uint32_t)n + (s - q * (uint32_t)ld));
+  } else {
+    const uint32_t word = links.code[r * ld + i];
+    const int32_t e = (int32_t)(word / kLinkPage);
+    adj[r * n + i] = e >= kLinkPages
+                         ? opp(r + 1) * n + i
+                         : (r + 1) * n + links.pages[32 * (i / kLinkTile) + e] + (int32_t)(word % kLinkPage);
+  }
 }
 
 }  // namespace
+
+int64_t one_wave_cells() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return 4 * (int64_t)sms * kSweepThreads;
+}
 
 int make_key_space(const int32_t dims[3], const lbm_ordering& ord, bool clamp_blocks,
                    KeySpace* ks) {
@@ -320,7 +395,7 @@ int make_key_space(const int32_t dims[3], const lbm_ordering& ord, bool clamp_bl
 }
 
 int public_links(const lbm_sparse* sp_c, const int32_t** out) {
-  // logically const: the public links are a cached view of adj_ld
+  // logically const: the public links are a cached view of the steps' links
   lbm_sparse* sp = const_cast<lbm_sparse*>(sp_c);
   if (!sp->adj) {
     const cudaStream_t stream = sp->stream;
@@ -333,7 +408,7 @@ int public_links(const lbm_sparse* sp_c, const int32_t** out) {
     }
     if (sp->n > 0)
       public_links_kernel<<<dim3((unsigned)((sp->n + 255) / 256), 18), 256, 0, stream>>>(
-          sp->adj_ld, (int32_t)sp->ld, (int32_t)sp->n, adj);
+          state_links(sp), (int32_t)sp->ld, (int32_t)sp->n, adj);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) {
@@ -388,7 +463,7 @@ extern "C" int lbm_build_sparse(const uint8_t* flags, const int32_t dims[3], lbm
   // scratch: tile counts, tile offsets, total, error flag
   uint32_t* counts = nullptr;
   int64_t* offsets = nullptr;
-  int64_t* scal = nullptr;  // [0] total, [1] bad-flag word
+  int64_t* scal = nullptr;  // [0] total, [1] bad-flag word, [2] short links overflow
   uint8_t* flags_copy = nullptr;
   lbm_sparse* sp = new lbm_sparse{};
   sp->magic = kMagicSparse;
@@ -406,6 +481,8 @@ extern "C" int lbm_build_sparse(const uint8_t* flags, const int32_t dims[3], lbm
       release(sp->inv);
       release(sp->adj);
       release(sp->adj_ld);
+      release(sp->code);
+      release(sp->pages);
       delete sp;
     }
     cudaStreamSynchronize(stream);
@@ -413,12 +490,12 @@ extern "C" int lbm_build_sparse(const uint8_t* flags, const int32_t dims[3], lbm
   };
   if (dev_alloc(&counts, sizeof(uint32_t) * ntiles, stream, true) != cudaSuccess ||
       dev_alloc(&offsets, sizeof(int64_t) * ntiles, stream, true) != cudaSuccess ||
-      dev_alloc(&scal, sizeof(int64_t) * 2, stream, true) != cudaSuccess ||
+      dev_alloc(&scal, sizeof(int64_t) * 3, stream, true) != cudaSuccess ||
       dev_alloc(&sp->inv, sizeof(int32_t) * box, stream, true) != cudaSuccess) {
     cudaGetLastError();
     return cleanup(fail(LBM_ENOMEM, "device allocation failed (box %lld cells)", (long long)box));
   }
-  if (cudaMemsetAsync(scal, 0, sizeof(int64_t) * 2, stream) != cudaSuccess)
+  if (cudaMemsetAsync(scal, 0, sizeof(int64_t) * 3, stream) != cudaSuccess)
     return cleanup(cuda_fail(cudaGetLastError(), "cudaMemsetAsync"));
   const uint8_t* flags_dev = flags;
   if (on_host) {
@@ -457,10 +534,26 @@ extern "C" int lbm_build_sparse(const uint8_t* flags, const int32_t dims[3], lbm
   sp->n = n;
   sp->ld = ld;
   const size_t nn = (size_t)(n > 0 ? n : 1);
-  // the links in the state layout; they are the public ones when ld == n
-  int32_t** links = ld == n ? &sp->adj : &sp->adj_ld;
-  if (dev_alloc(&sp->cells, sizeof(int32_t) * nn, stream, true) != cudaSuccess ||
-      dev_alloc(links, sizeof(int32_t) * 18 * (size_t)(ld > 0 ? ld : 1), stream, true) != cudaSuccess) {
+  // Lists of more than two waves take short links.  A smaller list's steps run
+  // from L2, where bytes count less than the decoding.  MFLUP/s with short /
+  // 32-bit links: 29,479 cells FP64 storage 8,148 / 8,890, FP32S 17,590 /
+  // 17,853, FP16S 18,730 / 18,446; 221,119 cells FP64 storage 19,623 / 21,163,
+  // FP32S 37,045 / 43,126, FP16S 36,547 / 44,828;
+  // 413,546 cells FP64 storage 16,411 / 14,675, FP32S 43,166 / 38,031.
+  const bool brief = n > 2 * one_wave_cells();
+  const auto alloc_wide = [&]() {   // they are the public links when ld == n
+    int32_t** links = ld == n ? &sp->adj : &sp->adj_ld;
+    return dev_alloc(links, sizeof(int32_t) * 18 * (size_t)(ld > 0 ? ld : 1), stream, true);
+  };
+  cudaError_t ea = dev_alloc(&sp->cells, sizeof(int32_t) * nn, stream, true);
+  if (brief) {
+    if (ea == cudaSuccess) ea = dev_alloc(&sp->code, sizeof(uint16_t) * 18 * (size_t)ld, stream, true);
+    if (ea == cudaSuccess)
+      ea = dev_alloc(&sp->pages, sizeof(int32_t) * 32 * (size_t)(ld / kLinkTile), stream, true);
+  } else if (ea == cudaSuccess) {
+    ea = alloc_wide();
+  }
+  if (ea != cudaSuccess) {
     cudaGetLastError();
     return cleanup(fail(LBM_ENOMEM, "device allocation failed (%lld fluid cells)", (long long)n));
   }
@@ -470,15 +563,38 @@ extern "C" int lbm_build_sparse(const uint8_t* flags, const int32_t dims[3], lbm
   else
     tile_scatter_kernel<<<(unsigned)ntiles, kTileThreads, 0, stream>>>(ks, flags_dev, offsets,
                                                                       sp->cells, sp->inv);
-  if (n > 0) {
-    const int threads = 256;
-    adjacency_kernel<<<(unsigned)((n + threads - 1) / threads), threads, 0, stream>>>(
-        dims[0], dims[1], dims[2], ord.periodic, sp->cells, sp->inv, *links, (int32_t)n,
-        (int32_t)ld);
+  const auto write_wide = [&]() {
+    if (n == 0) return;
+    adjacency_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(
+        dims[0], dims[1], dims[2], ord.periodic, sp->cells, sp->inv,
+        ld == n ? sp->adj : sp->adj_ld, (int32_t)n, (int32_t)ld);
+  };
+  if (brief) {
+    const unsigned tiles = (unsigned)(ld / kLinkTile);
+    short_links_kernel<<<(tiles + 7) / 8, 256, 0, stream>>>(
+        dims[0], dims[1], dims[2], ord.periodic, sp->cells, sp->inv, (int32_t)n, (int32_t)ld,
+        sp->code, sp->pages, (int32_t*)(scal + 2));
+    e = cudaMemcpyAsync(host_scal, scal + 2, sizeof(int64_t), cudaMemcpyDeviceToHost, stream);
+  } else {
+    write_wide();
   }
-  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-  if (e != cudaSuccess) return cleanup(cuda_fail(e, "sparse assembly: scatter/adjacency"));
+  if (e == cudaSuccess && brief && host_scal[0] != 0) {
+    // a tile's neighbours lie in more than kLinkPages pages
+    release(sp->code);
+    release(sp->pages);
+    sp->code = nullptr;
+    sp->pages = nullptr;
+    if (alloc_wide() != cudaSuccess) {
+      cudaGetLastError();
+      return cleanup(fail(LBM_ENOMEM, "device allocation failed (%lld fluid cells)", (long long)n));
+    }
+    write_wide();
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  }
+  if (e != cudaSuccess) return cleanup(cuda_fail(e, "sparse assembly: scatter/links"));
   *out = sp;
   return cleanup(LBM_OK);
 }

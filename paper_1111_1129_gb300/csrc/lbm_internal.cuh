@@ -265,15 +265,18 @@ struct lbm_sparse {
   int64_t n;
   int32_t* cells;  // [n]
   int32_t* inv;    // [box]
-  // [18 * n], source slot q n + m (the layout lbm_sparse_info presents).
-  // When ld != n the assembly writes adj_ld only, and adj is derived from
-  // it on first request (public_links); null until then.
+  // [18 * n], source slot q n + m (the layout lbm_sparse_info presents):
+  // derived from the links below on first request (public_links), null until
+  // then, except where it serves as adj_ld.
   int32_t* adj;
   // Row stride of the state arrays: n rounded up to kRowAlign (a batch: its
-  // padded total).  adj_ld holds the links in that layout, rows of ld
-  // entries naming slot r ld + m; null when ld == n (adj serves).
+  // padded total).  The links the steps read name slots r ld + m, in one of
+  // two forms: short links (code, pages; see lbm::Links), or 32-bit ones in
+  // rows of ld, adj_ld (null when ld == n: adj serves).
   int64_t ld;
   int32_t* adj_ld;
+  uint16_t* code;
+  int32_t* pages;
   cudaStream_t stream;
 };
 
@@ -287,10 +290,32 @@ namespace lbm {
 // on every other row, and every form's warp accesses straddle one more line.
 constexpr int64_t kRowAlign = 64;
 inline int64_t row_stride(int64_t n) { return (n + kRowAlign - 1) / kRowAlign * kRowAlign; }
-// The links the sweeps of a state on sp read: rows of sp->ld entries.
-inline const int32_t* state_links(const lbm_sparse* sp) { return sp->adj_ld ? sp->adj_ld : sp->adj; }
-// The public links of sp (*out may be null), built from adj_ld on the first
-// request and kept (one kernel on sp's stream, which is then synchronised).
+
+// The links a step reads: 32-bit slots r ld + m in rows of ld (`wide`), or
+// short links (wide null).  Those hold each link in 16 bits, 18 rows of ld
+// codes.  Cells are taken in tiles of kLinkTile; a tile lists the pages (runs
+// of kLinkPage cells of the list) its neighbours lie in, at most
+// kLinkPages of them, in 32 entries `pages + 32 tile`, and a code is an entry
+// (5 bits) and the neighbour's place in that page (11 bits).  Entry e holds
+// the page's first cell, so that the slot is
+//   r ld + pages[32 tile + (code >> 11)] + (code & 2047);
+// entries 30 and 31 hold the tile's first cell plus and minus ld, so that a
+// link bounced back at cell i, slot opp(r) ld + i, is entry 30 (r odd) or 31
+// (r even) with i's place in the tile: no case of its own.
+// A step then reads 38 bytes of links per cell instead of 72.
+struct Links {
+  const int32_t* wide;
+  const uint16_t* code;
+  const int32_t* pages;
+};
+constexpr int32_t kLinkTile = 64, kLinkPage = 2048, kLinkPages = 30;
+static_assert(kRowAlign % kLinkTile == 0, "whole tiles in a row");
+inline Links state_links(const lbm_sparse* sp) {
+  if (sp->code) return Links{nullptr, sp->code, sp->pages};
+  return Links{sp->adj_ld ? sp->adj_ld : sp->adj, nullptr, nullptr};
+}
+// The public links of sp (*out may be null), built from those the steps read
+// on the first request and kept (one kernel on sp's stream, which is then synchronised).
 int public_links(const lbm_sparse* sp, const int32_t** out);
 }  // namespace lbm
 
@@ -398,7 +423,7 @@ struct lbm_state {
   double* partials;    // [nblocks * kWarpsPerBlock * 4] FP64 warp sums of the last step,
                        // then [nblocks * 4] room for the group values of lbm_reduce_flux
   int64_t nblocks;
-  bool one_wave;       // nblocks <= 4 x SMs: plain FP32/16-bit steps load links first
+  bool one_wave;       // at most one_wave_cells(): plain FP32/16-bit steps load links first
   double* red_dev;     // [4] final sums
   double* red_host;    // [4] pinned
   int64_t steps;
@@ -411,6 +436,9 @@ struct lbm_state {
 };
 
 namespace lbm {
+// Cells of one wave of the FP32 and 16-bit sweeps on the current device, at
+// their 4 resident 256-thread blocks per SM (0 if the device cannot be asked).
+int64_t one_wave_cells();
 void free_state(lbm_state* st);
 void free_sparse(lbm_sparse* sp);
 void free_adjoint(lbm_adjoint* ad);

@@ -434,6 +434,53 @@ __device__ __forceinline__ void load_links(const int32_t* __restrict__ adj, int3
   for (int q = 0; q < 18; ++q) idx[q] = ld_nc(adj + q * ld + i);
 }
 
+__device__ __forceinline__ uint32_t ld_nc_u32(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.nc" LBM_LD_HINT ".u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+
+// Slot named by short link `word` of row q > 0, given this lane's entry of
+// the tile's pages.  A shuffle takes the lane modulo 32, so bits above the
+// word's entry do no harm.
+__device__ __forceinline__ int32_t short_slot(int q, int32_t ld, int32_t entry, uint32_t word) {
+  return __shfl_sync(0xffffffffu, entry, (int)(word / kLinkPage)) +
+         (int32_t)(word % kLinkPage) + q * ld;
+}
+__device__ __forceinline__ int32_t page_entry(const Links& links, int32_t i) {
+  return ld_nc(links.pages + 32 * (i / kLinkTile) + (int32_t)(threadIdx.x & 31));
+}
+
+// The 18 slots cell i of n pulls from.  Short links are decoded by the whole
+// warp, whose cells lie in one tile: every lane of a warp with a cell below
+// ld takes part (idx of cells from n on names slots in range, not links).
+// All codes are requested before the first is decoded.
+template <bool SHORT>
+__device__ __forceinline__ void load_links(const Links& links, int32_t n, int32_t ld, int32_t i,
+                                           int32_t idx[18]) {
+  if constexpr (SHORT) {
+    if (i >= ld) return;
+    const unsigned short* code = reinterpret_cast<const unsigned short*>(links.code) + i;
+    uint32_t word[18];
+#pragma unroll
+    for (int q = 0; q < 18; ++q) word[q] = ld_nc(code + q * ld);
+    const int32_t entry = page_entry(links, i);
+#pragma unroll
+    for (int q = 0; q < 18; ++q) idx[q] = short_slot(q + 1, ld, entry, word[q]);
+  } else {
+    if (i < n) load_links(links.wide, ld, i, idx);
+  }
+}
+
+// One link of cell i, by itself (q > 0).
+template <bool SHORT>
+__device__ __forceinline__ int32_t one_link(const Links& links, int32_t ld, int32_t i, int q) {
+  if constexpr (!SHORT) return __ldg(links.wide + (q - 1) * ld + i);
+  const uint32_t word = __ldg(links.code + (q - 1) * ld + i);
+  return q * ld + __ldg(links.pages + 32 * (i / kLinkTile) + (int32_t)(word / kLinkPage)) +
+         (int32_t)(word % kLinkPage);
+}
+
 // The 19 pulled values of cell i, given its adjacency entries.
 template <int PREC>
 __device__ __forceinline__ void pull(const typename Form<PREC>::S* __restrict__ src,
@@ -515,10 +562,11 @@ constexpr int sweep_launch_min_blocks() {
 // after.  On a grid of one wave (the 32x32x64 bed) that made the FP32 and
 // 16-bit steps 15-17% faster; on the 1024x256x256 bed it cost the FP16 step
 // 0.9%, and the fixed-point kernel spilled with it.
-template <int PREC, bool DAMPED, int RED, bool LINKS_FIRST = false>
+// SHORT: the links are short ones.
+template <int PREC, bool DAMPED, int RED, bool SHORT = false, bool LINKS_FIRST = false>
 __global__ void __launch_bounds__(kSweepThreads, sweep_launch_min_blocks<PREC, RED>())
     sweep_kernel(const typename Form<PREC>::S* __restrict__ src,
-                 typename Form<PREC>::S* __restrict__ dst, const int32_t* __restrict__ adj,
+                 typename Form<PREC>::S* __restrict__ dst, Links links,
                  int32_t n, int32_t ld, Coef<typename Form<PREC>::C> k,
                  const typename Form<PREC>::C* __restrict__ alpha, double* __restrict__ partials) {
   using C = typename Form<PREC>::C;
@@ -527,7 +575,7 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_launch_min_blocks<PREC, R
   int32_t idx[18];
   int32_t z = 0;
   if constexpr (!LINKS_FIRST) z = prior_step_done();
-  if (i < n) load_links(adj, ld, i, idx);
+  load_links<SHORT>(links, n, ld, i, idx);
   if constexpr (LINKS_FIRST) z = prior_step_done();
   if (i < n) {
     C g[19];
@@ -555,64 +603,84 @@ __device__ __forceinline__ uint32_t c_to_bits(float v, float scale) {
   else return __bfloat16_as_ushort(__float2bfloat16_rn(v * scale));
 }
 
-// ---- two adjacent cells per thread (16-bit forms) ----------------------------
-// A thread updates cells i and i + 1 (i even), so a warp covers 64
-// consecutive cells and has twice the cells in flight at the same 64
-// registers (4 blocks per SM).  The two accesses of a row are issued back to
-// back -- both cells' links, both pulls, and, after both collisions, both
-// stores -- so each pair lands on the same sectors at once and L1 and L2
-// merge them.  Loads stay scalar; a row whose element q ld + i is even
-// (every row: the row stride ld is a multiple of kRowAlign) takes the pair's
-// two stores as one 4-byte store, which cuts the store instructions the LSU
-// queue holds.  FP16 on the 1024x256x256 bed (N odd), MFLUP/s: with rows of
-// stride N, alternating runs: one cell per thread 40,579-40,653; pair, all
-// scalar 42,434-42,453; pair with the 4-byte stores on the even rows
-// 43,307-43,376.  With every row aligned (this kernel) 45,779-45,784.
-// Measured slower, on rows of stride N: 4-byte stores on the odd rows too,
-// built with a lane shuffle, 41,923; one 4-byte load for both pulls where they share a word 29,135;
-// 8-byte link loads on the aligned rows 29,844-30,936 (with and without the
-// L2 hint, non-coherent or coherent; with registers to spare, 78 at 3 blocks
-// per SM, 25,215 against 41,622 for scalar loads at that occupancy, so not
-// register pressure); link rows through bulk copies into
-// shared memory, completed on an mbarrier 36,780; three or four cells per
-// thread 33,154 / 28,450; cells i and i + 32 of a warp's 64 40,189; links
-// loaded before the wait for the previous step 37,263; write-back stores
-// 42,277 (against 42,447); 2-byte rest-row loads 42,249; 128-thread blocks
-// 41,209.  The per-cell arithmetic is that of sweep_kernel, so results are
-// bit-identical to it.
-#ifndef LBM_PAIR_SWEEP
-#define LBM_PAIR_SWEEP 1
-#endif
-#ifndef LBM_PAIR_REST_U32
-#define LBM_PAIR_REST_U32 1
-#endif
+// ---- two adjacent cells per thread ------------------------------------------
+// A thread updates cells i and i + 1 (i even), so a warp covers 64 consecutive
+// cells -- one tile of short links -- and has twice the cells in flight.
+// One 4-byte load brings both cells' codes of a row, and one store both
+// results (every row is aligned: the row stride is a multiple of kRowAlign);
+// the pulls stay scalar, back to back, so that each pair lands on the same
+// sectors and L1 merges them.  The per-cell arithmetic is that of
+// sweep_kernel, so results are bit-identical to it.
+//
+// What bounds them: DRAM bytes in FP32 (190 per update, 38 of them links), the
+// latency of the two dependent round trips (codes, then pulls) in the 16-bit
+// forms.  1024x256x256 bed, MFLUP/s, lexicographic / 8^3 blocked order:
+//   FP32S  one cell, 32-bit links 31,444 / 30,249; one cell, short links
+//          32,380 / 31,396; pair 36,746 / 35,079 (1.05 of the copy rate)
+//   FP16S  pair, 32-bit links 45,648 / 43,751; pair, short links
+//          51,409 / 49,378 (0.88)
+// Launch shapes: FP32 in 128-thread blocks at 6 per SM (80 registers); 7 per
+// SM 36,786 / 35,061, 5 36,457 / 34,880, 256 threads x 3 36,596 and x 4
+// (64 registers, spills) 34,956 in lexicographic order.  16-bit forms in
+// 256-thread blocks at 4 per SM (64 registers); 128 threads x 8
+// 50,608 / 46,973, x 6 50,123 / 47,052.  Measured slower in the 16-bit forms,
+// with 32-bit links on rows of stride N (pair 43,376): 4-byte stores on
+// misaligned rows, built with a lane shuffle, 41,923; one 4-byte load for both
+// pulls where they share a word 29,135; link rows through bulk copies into
+// shared memory 36,780; three or four cells per thread 33,154 / 28,450; cells
+// i and i + 32 of a warp's 64 40,189; links loaded before the wait for the
+// previous step 37,263; write-back stores 42,277.  A list whose tiles meet too
+// many pages for short links takes one cell per thread.
 #ifndef LBM_PAIR_THREADS
 #define LBM_PAIR_THREADS 256
 #endif
-constexpr int kPairThreads = LBM_PAIR_THREADS;
+#ifndef LBM_PAIR_MIN_BLOCKS
+#define LBM_PAIR_MIN_BLOCKS 4
+#endif
+#ifndef LBM_PAIR32_THREADS
+#define LBM_PAIR32_THREADS 128
+#endif
+#ifndef LBM_PAIR32_MIN_BLOCKS
+#define LBM_PAIR32_MIN_BLOCKS 6
+#endif
+constexpr int kPairThreads = LBM_PAIR_THREADS, kPair32Threads = LBM_PAIR32_THREADS;
 
-__device__ __forceinline__ uint32_t ld_nc_u32(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.global.nc" LBM_LD_HINT ".u32 %0, [%1];" : "=r"(v) : "l"(p));
-  return v;
+// The short links of cells i, i + 1 (i even), both in one word, low half i.
+__device__ __forceinline__ void load_pair_links(const Links& links, int32_t ld, int32_t i,
+                                                uint32_t word[18], int32_t& entry) {
+#pragma unroll
+  for (int q = 0; q < 18; ++q)
+    word[q] = ld_nc_u32(reinterpret_cast<const uint32_t*>(links.code + q * ld + i));
+  entry = page_entry(links, i);
 }
 
-// Pulls, both collisions and the stores of the pair (i, i + 1), given their
-// links a (cell i) and b (cell i + 1); dst rows of stride ld.
 template <int PREC, bool DAMPED>
-__device__ __forceinline__ void pair_body(const typename Form<PREC>::S* __restrict__ src,
-                                          typename Form<PREC>::S* __restrict__ dst, int32_t ld,
-                                          const Coef<float>& k, const float* __restrict__ alpha,
-                                          int32_t i, bool two, bool odd_ld, const int32_t a[18],
-                                          const int32_t b[18]) {
+__global__ void __launch_bounds__(kPairThreads, LBM_PAIR_MIN_BLOCKS)
+    sweep_pair_kernel(const typename Form<PREC>::S* __restrict__ src,
+                      typename Form<PREC>::S* __restrict__ dst, Links links, int32_t n,
+                      int32_t ld, Coef<float> k, const float* __restrict__ alpha) {
+  static_assert(PREC == LBM_F16S || PREC == LBM_BF16S, "16-bit forms only");
+  const int32_t z = prior_step_done();
+  const int32_t i = 2 * (int32_t)(blockIdx.x * kPairThreads + threadIdx.x) + z;
+  if (i >= ld) return;   // whole warps: their 64 cells are one tile of links
+  const bool two = i + 1 < n;   // false for the last cell of an odd-length list, and past it
   const unsigned short* src16 = reinterpret_cast<const unsigned short*>(src);
+  uint32_t word[18];
+  int32_t entry;
+  load_pair_links(links, ld, i, word, entry);
+  int32_t a[18], b[18];
+#pragma unroll
+  for (int q = 0; q < 18; ++q) {
+    a[q] = short_slot(q + 1, ld, entry, word[q]);
+    b[q] = short_slot(q + 1, ld, entry, word[q] >> 16);
+  }
+  if (i >= n) return;
   // pulled values, packed: low half cell i, high half cell i + 1
   uint32_t g[19];
-  if (LBM_PAIR_REST_U32 && two) {   // the rest row is aligned at even i
+  if (two) {   // the rest row is aligned at even i
     g[0] = ld_nc_u32(reinterpret_cast<const uint32_t*>(src) + (i >> 1));
   } else {
     g[0] = ld_nc(src16 + i);
-    if (two) g[0] |= (uint32_t)ld_nc(src16 + i + 1) << 16;
   }
 #pragma unroll
   for (int q = 0; q < 18; ++q) {
@@ -638,50 +706,65 @@ __device__ __forceinline__ void pair_body(const typename Form<PREC>::S* __restri
   unsigned short* dst16 = reinterpret_cast<unsigned short*>(dst);
 #pragma unroll
   for (int q = 0; q < 19; ++q) {
-    const int32_t e = q * ld + i;
-    if (two && !(odd_ld && (q & 1))) {   // element e is even: one 4-byte store of the pair
-      asm volatile("st.global.cs.u32 [%0], %1;" ::"l"(dst16 + e), "r"(out[q]) : "memory");
-    } else {
-      st_cs(dst16 + e, (unsigned short)(out[q] & 0xffffu));
-      if (two) st_cs(dst16 + e + 1, (unsigned short)(out[q] >> 16));
-    }
+    const int32_t e = q * ld + i;   // even: one 4-byte store of the pair
+    if (two) asm volatile("st.global.cs.u32 [%0], %1;" ::"l"(dst16 + e), "r"(out[q]) : "memory");
+    else st_cs(dst16 + e, (unsigned short)(out[q] & 0xffffu));
   }
 }
 
+// The same for the FP32 forms.
 template <int PREC, bool DAMPED>
-__global__ void __launch_bounds__(kPairThreads, 4 * 256 / kPairThreads)
-    sweep_pair_kernel(const typename Form<PREC>::S* __restrict__ src,
-                      typename Form<PREC>::S* __restrict__ dst, const int32_t* __restrict__ adj,
-                      int32_t n, int32_t ld, Coef<float> k, const float* __restrict__ alpha) {
-  static_assert(PREC == LBM_F16S || PREC == LBM_BF16S, "16-bit forms only");
+__global__ void __launch_bounds__(kPair32Threads, LBM_PAIR32_MIN_BLOCKS)
+    sweep_pair32_kernel(const float* __restrict__ src, float* __restrict__ dst, Links links,
+                        int32_t n, int32_t ld, Coef<float> k, const float* __restrict__ alpha) {
+  static_assert(PREC == LBM_F32 || PREC == LBM_F32S, "FP32 forms only");
   const int32_t z = prior_step_done();
-  const int32_t i = 2 * (int32_t)(blockIdx.x * kPairThreads + threadIdx.x) + z;
-  if (i >= n) return;
-  const bool two = i + 1 < n;   // false only for the last cell of an odd-length list
-  const bool odd_ld = (ld & 1) != 0;
-  int32_t a[18], b[18];
+  const int32_t i = 2 * (int32_t)(blockIdx.x * kPair32Threads + threadIdx.x) + z;
+  if (i >= ld) return;   // whole warps
+  const bool two = i + 1 < n;
+  uint32_t word[18];
+  int32_t entry;
+  load_pair_links(links, ld, i, word, entry);
+  float g[2][19];
+  if (i < n) g[0][0] = ld_nc(src + i);
+  if (two) g[1][0] = ld_nc(src + i + 1);
 #pragma unroll
   for (int q = 0; q < 18; ++q) {
-    const int32_t* p = adj + q * ld + i;
-    a[q] = ld_nc(p);
-    b[q] = two ? ld_nc(p + 1) : 0;
+    const int32_t a = short_slot(q + 1, ld, entry, word[q]);
+    const int32_t b = short_slot(q + 1, ld, entry, word[q] >> 16);
+    if (i < n) g[0][q + 1] = ld_nc(src + a);
+    if (two) g[1][q + 1] = ld_nc(src + b);
   }
-  pair_body<PREC, DAMPED>(src, dst, ld, k, alpha, i, two, odd_ld, a, b);
+  if (i >= n) return;
+  float rho, u[3];
+  collide<float, DAMPED>(g[0], k, DAMPED ? ld_nc(alpha + i) : 0.f, rho, u);
+  if (two) {
+    collide<float, DAMPED>(g[1], k, DAMPED ? ld_nc(alpha + i + 1) : 0.f, rho, u);
+#pragma unroll
+    for (int q = 0; q < 19; ++q)
+      asm volatile("st.global.cs.v2.f32 [%0], {%1, %2};" ::"l"(dst + q * ld + i), "f"(g[0][q]),
+                   "f"(g[1][q]) : "memory");
+  } else {
+#pragma unroll
+    for (int q = 0; q < 19; ++q) st_cs(dst + q * ld + i, g[0][q]);
+  }
 }
 
 // Per-cell moments of the collision that a step from `src` performs (rows
 // of stride ld; rho_out [n], u_out [3][n]).
-template <int PREC, bool DAMPED>
+template <int PREC, bool DAMPED, bool SHORT>
 __global__ void __launch_bounds__(kSweepThreads)
-    moments_kernel(const typename Form<PREC>::S* __restrict__ src, const int32_t* __restrict__ adj,
-                   int32_t n, int32_t ld, Coef<typename Form<PREC>::C> k,
+    moments_kernel(const typename Form<PREC>::S* __restrict__ src, Links links, int32_t n,
+                   int32_t ld, Coef<typename Form<PREC>::C> k,
                    const typename Form<PREC>::C* __restrict__ alpha, double* __restrict__ rho_out,
                    double* __restrict__ u_out) {
   using C = typename Form<PREC>::C;
   const int32_t i = blockIdx.x * kSweepThreads + threadIdx.x;
+  int32_t idx[18];
+  load_links<SHORT>(links, n, ld, i, idx);
   if (i >= n) return;
   C g[19];
-  gather<PREC>(src, adj, ld, i, k.inv_scale, g);
+  pull<PREC>(src, idx, i, k.inv_scale, g);
   C rho, u[3];
   collide<C, DAMPED>(g, k, DAMPED ? alpha[i] : C(0), rho, u);
   rho_out[i] = Form<PREC>::kShifted ? 1.0 + (double)rho : (double)rho;

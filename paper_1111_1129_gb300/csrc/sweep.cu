@@ -2,9 +2,10 @@
 // (Sec. 1: TRT on D3Q19; Sec. 2: sparse representation with implicit bounce
 // back; Sec. 7: pull scheme, structure of arrays, nontemporal stores).
 //
-// One thread updates one fluid cell per step (two adjacent cells in the
-// plain steps of the 16-bit forms, sweep_pair_kernel):
-//   gather   g_0 = f[n], g_i = f[adj[i-1][n]]     (pull through the list)
+// One thread updates one fluid cell per step (two adjacent cells in the plain
+// 16-bit and FP32 steps of larger lists, sweep_pair_kernel):
+//   gather   g_0 = f[n], g_i = f[adj[i-1][n]]     (pull through the list,
+//            whose links the steps of larger lists read in 16 bits, lbm::Links)
 //   collide  TRT with body force and Brinkman damping, written on the nine
 //            (c, -c) pairs: with s = g_a + g_b, d = g_a - g_b,
 //              f*_a = P + Q,  f*_b = P - Q,
@@ -25,7 +26,7 @@
 // rho - 1, because w_q is the equilibrium of rho = 1, u = 0.
 //
 // A state's PDF rows, and the link rows its steps read, have the stride
-// sp->ld (N rounded up to 64), so that every row starts on a 128-byte
+// sp->ld (N rounded up to 64), so that every row of PDFs starts on a 128-byte
 // boundary; the links name slots r ld + m.  Host-facing copies (set/get
 // PDFs, moments) use the plain [19][N] layout.
 #include <cuda_bf16.h>
@@ -136,57 +137,61 @@ bool valid_state(const lbm_state* st) { return st && st->magic == kMagicState; }
 
 namespace {
 
+// One step of a state from src to dst.  The lists that have short links take
+// two adjacent cells per thread in their plain FP32 and 16-bit steps; a list
+// of one wave loads its links before the wait.
+template <int PREC, bool DAMPED, bool SHORT>
+cudaError_t launch_step(const lbm_state* st, const typename Form<PREC>::S* src,
+                        typename Form<PREC>::S* dst, const Links& links,
+                        const Coef<typename Form<PREC>::C>& k, cudaStream_t stream, bool chained,
+                        bool reduce) {
+  const int32_t n = (int32_t)st->sp->n, ld = (int32_t)st->sp->ld;
+  const unsigned grid = (unsigned)st->nblocks;
+  const auto* alpha = (const typename Form<PREC>::C*)st->alpha;
+  if (reduce)
+    return launch_sweep(sweep_kernel<PREC, DAMPED, kWarpSums, SHORT>, grid, stream, chained, src,
+                        dst, links, n, ld, k, alpha, st->partials);
+  if constexpr (SHORT && (PREC == LBM_F16S || PREC == LBM_BF16S)) {
+    constexpr int64_t cells = 2 * (int64_t)kPairThreads;
+    return launch_chained(sweep_pair_kernel<PREC, DAMPED>, (unsigned)((n + cells - 1) / cells),
+                          (unsigned)kPairThreads, stream, chained, src, dst, links, n, ld, k, alpha);
+  } else if constexpr (SHORT && (PREC == LBM_F32 || PREC == LBM_F32S)) {
+    constexpr int64_t cells = 2 * (int64_t)kPair32Threads;
+    return launch_chained(sweep_pair32_kernel<PREC, DAMPED>, (unsigned)((n + cells - 1) / cells),
+                          (unsigned)kPair32Threads, stream, chained, src, dst, links, n, ld, k, alpha);
+  } else {
+    if constexpr (!SHORT && PREC != LBM_F64)
+      if (st->one_wave)
+        return launch_sweep(sweep_kernel<PREC, DAMPED, kNoReduce, false, true>, grid, stream,
+                            chained, src, dst, links, n, ld, k, alpha, st->partials);
+    return launch_sweep(sweep_kernel<PREC, DAMPED, kNoReduce, SHORT>, grid, stream, chained, src,
+                        dst, links, n, ld, k, alpha, st->partials);
+  }
+}
+
 template <int PREC>
 int launch_steps(lbm_state* st, int32_t n_steps, double wp, double wm, const double F[3],
                  cudaStream_t stream, bool reduce_last) {
-  using S = typename Form<PREC>::S;
-  using C = typename Form<PREC>::C;
-  const int32_t n = (int32_t)st->sp->n;
-  const int32_t ld = (int32_t)st->sp->ld;
-  if constexpr (PREC == LBM_F64X) return launch_steps_fx(st, n_steps, wp, wm, F, stream, reduce_last);
-  const Coef<C> k = make_coef<C>(wp, wm, F, st->scale_exp);
-  const unsigned grid = (unsigned)st->nblocks;
-  const C* alpha = (const C*)st->alpha;
-  // the 16-bit forms take two adjacent cells per thread in their plain steps
-  // on grids of more than one wave
-  constexpr bool kPairForm = LBM_PAIR_SWEEP && (PREC == LBM_F16S || PREC == LBM_BF16S);
-  constexpr int64_t kPairCells = 2 * (int64_t)kPairThreads;
-  const unsigned grid_pair = (unsigned)((n + kPairCells - 1) / kPairCells);
-  for (int32_t t = 0; t < n_steps; ++t) {
-    const S* src = (const S*)st->buf[st->cur];
-    S* dst = (S*)st->buf[st->cur ^ 1];
-    const bool last = reduce_last && t == n_steps - 1;
-    if (n > 0) {
-      const int32_t* adj = state_links(st->sp);
+  if constexpr (PREC == LBM_F64X) {
+    return launch_steps_fx(st, n_steps, wp, wm, F, stream, reduce_last);
+  } else {
+    using S = typename Form<PREC>::S;
+    const auto k = make_coef<typename Form<PREC>::C>(wp, wm, F, st->scale_exp);
+    const Links links = state_links(st->sp);
+    const auto step = links.wide ? (st->alpha ? launch_step<PREC, true, false> : launch_step<PREC, false, false>)
+                                 : (st->alpha ? launch_step<PREC, true, true> : launch_step<PREC, false, true>);
+    for (int32_t t = 0; t < n_steps; ++t) {
       // Steps in FP64 arithmetic are not chained: a chained grid's blocks are
       // placed while the previous grid still holds its SMs, which packs
       // them onto fewer SMs, and these steps are bound by each SM's FP64
       // rate (32x32x64 bed: 2,333 against 2,580 MFLUP/s unchained).
-      constexpr bool kMemoryBound = PREC != LBM_F64 && PREC != LBM_F64X;
-      const bool chained = kMemoryBound && t > 0;
-      // a grid of one wave loads its links before the wait (sweep_kernel)
-      const bool links_first = kMemoryBound && st->one_wave && !last;
-      if constexpr (kPairForm) {
-        if (!last && !st->one_wave) {
-          if (alpha) LBM_CUDA_TRY(launch_chained(sweep_pair_kernel<PREC, true>, grid_pair, (unsigned)kPairThreads, stream, chained, src, dst, adj, n, ld, k, alpha));
-          else LBM_CUDA_TRY(launch_chained(sweep_pair_kernel<PREC, false>, grid_pair, (unsigned)kPairThreads, stream, chained, src, dst, adj, n, ld, k, alpha));
-          st->cur ^= 1;
-          continue;
-        }
-      }
-      if (alpha) {
-        if (last) LBM_CUDA_TRY(launch_sweep(sweep_kernel<PREC, true, kWarpSums>, grid, stream, chained, src, dst, adj, n, ld, k, alpha, st->partials));
-        else if (links_first) LBM_CUDA_TRY(launch_sweep(sweep_kernel<PREC, true, kNoReduce, kMemoryBound>, grid, stream, chained, src, dst, adj, n, ld, k, alpha, st->partials));
-        else LBM_CUDA_TRY(launch_sweep(sweep_kernel<PREC, true, kNoReduce>, grid, stream, chained, src, dst, adj, n, ld, k, alpha, st->partials));
-      } else {
-        if (last) LBM_CUDA_TRY(launch_sweep(sweep_kernel<PREC, false, kWarpSums>, grid, stream, chained, src, dst, adj, n, ld, k, alpha, st->partials));
-        else if (links_first) LBM_CUDA_TRY(launch_sweep(sweep_kernel<PREC, false, kNoReduce, kMemoryBound>, grid, stream, chained, src, dst, adj, n, ld, k, alpha, st->partials));
-        else LBM_CUDA_TRY(launch_sweep(sweep_kernel<PREC, false, kNoReduce>, grid, stream, chained, src, dst, adj, n, ld, k, alpha, st->partials));
-      }
+      if (st->sp->n > 0)
+        LBM_CUDA_TRY(step(st, (const S*)st->buf[st->cur], (S*)st->buf[st->cur ^ 1], links, k,
+                          stream, PREC != LBM_F64 && t > 0, reduce_last && t == n_steps - 1));
+      st->cur ^= 1;
     }
-    st->cur ^= 1;
+    return LBM_OK;
   }
-  return LBM_OK;
 }
 
 template <int PREC>
@@ -198,10 +203,11 @@ int launch_moments(const lbm_state* st, double* rho, double* u) {
   const Coef<C> k = make_coef<C>(st->last_wp, st->last_wm, st->last_force, st->scale_exp);
   const S* prev = (const S*)st->buf[st->cur ^ 1];
   const C* alpha = (const C*)st->alpha;
-  if (alpha)
-    moments_kernel<PREC, true><<<(unsigned)st->nblocks, kSweepThreads, 0, st->sp->stream>>>(prev, state_links(st->sp), n, (int32_t)st->sp->ld, k, alpha, rho, u);
-  else
-    moments_kernel<PREC, false><<<(unsigned)st->nblocks, kSweepThreads, 0, st->sp->stream>>>(prev, state_links(st->sp), n, (int32_t)st->sp->ld, k, alpha, rho, u);
+  const Links links = state_links(st->sp);
+  const auto kernel = links.wide ? (alpha ? moments_kernel<PREC, true, false> : moments_kernel<PREC, false, false>)
+                                 : (alpha ? moments_kernel<PREC, true, true> : moments_kernel<PREC, false, true>);
+  kernel<<<(unsigned)st->nblocks, kSweepThreads, 0, st->sp->stream>>>(
+      prev, links, n, (int32_t)st->sp->ld, k, alpha, rho, u);
   LBM_CUDA_TRY(cudaGetLastError());
   return LBM_OK;
 }
@@ -384,7 +390,7 @@ extern "C" int lbm_state_create(const lbm_sparse* sp, int32_t precision, int32_t
   if (!out) return fail(LBM_EINVAL, "out is NULL");
   *out = nullptr;
   if (!sp || sp->magic != kMagicSparse) return fail(LBM_EINVAL, "not a sparse handle");
-  if (sp->ld < sp->n || (sp->ld != sp->n && !sp->adj_ld))
+  if (sp->ld < sp->n || (sp->ld != sp->n && !sp->adj_ld && !sp->code))
     return fail(LBM_EINVAL, "sparse handle without a valid row layout");
   if (precision < LBM_F64 || precision > LBM_F64X)
     return fail(LBM_EINVAL, "unknown precision %d", precision);
@@ -399,14 +405,7 @@ extern "C" int lbm_state_create(const lbm_sparse* sp, int32_t precision, int32_t
   const int64_t n = sp->n;
   st->nblocks = (n + kSweepThreads - 1) / kSweepThreads;
   if (st->nblocks < 1) st->nblocks = 1;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    sms = 0;
-  }
-  // one wave at the 4 resident blocks per SM of the FP32 and 16-bit sweeps
-  st->one_wave = st->nblocks <= 4 * (int64_t)sms;
+  st->one_wave = n <= one_wave_cells();
   // rows of sp->ld elements; the padding slots past n are never read
   const size_t bytes = storage_bytes(precision) * 19 * (size_t)(sp->ld > 0 ? sp->ld : 1);
   const cudaStream_t stream = sp->stream;
@@ -716,10 +715,10 @@ extern "C" int lbm_step_f64_noalloc(const double* f_src_dev, double* f_dst_dev,
   const Coef<double> k = make_coef<double>(omega_plus, omega_minus, force, 0);
   if (alpha_dev)
     sweep_kernel<LBM_F64, true, kBlockSums><<<(unsigned)nblocks, kSweepThreads, 0, stream>>>(
-        f_src_dev, f_dst_dev, adj_dev, n, n, k, alpha_dev, partials);
+        f_src_dev, f_dst_dev, Links{adj_dev, nullptr, nullptr}, n, n, k, alpha_dev, partials);
   else
     sweep_kernel<LBM_F64, false, kBlockSums><<<(unsigned)nblocks, kSweepThreads, 0, stream>>>(
-        f_src_dev, f_dst_dev, adj_dev, n, n, k, nullptr, partials);
+        f_src_dev, f_dst_dev, Links{adj_dev, nullptr, nullptr}, n, n, k, nullptr, partials);
   final_sum_kernel<<<1, 1024, 0, stream>>>(partials, nblocks, sums_dev);
   LBM_CUDA_TRY(cudaGetLastError());
   return LBM_OK;

@@ -94,15 +94,16 @@ __device__ __forceinline__ int64_t wbits(int q) { return q == 0 ? kW0Bits : (q <
 __device__ __forceinline__ int64_t wexp(int q) { return q == 0 ? 0x3FD : (q <= 6 ? 0x3FA : 0x3F9); }
 __device__ __forceinline__ int wshift(int q) { return q == 0 ? 4 : (q <= 6 ? 1 : 0); }
 
-// Resident blocks of 256 threads per SM the register budget is fitted to:
-// on the 1024x256x256 bed 3 (80 registers) beat 2 (120 registers) by 15%
-// and 4 (64 registers, heavy spills) by 5%.  The reducing kernel, which
-// runs once per lbm_step call, is fitted to 3 as well: 1.98 ms per launch
-// there (2.19 ms at 2 blocks, 128 registers, and at 4, 64 registers with
-// 168 bytes spilled), against 1.80 ms for a plain step.
-#ifndef LBM_FX_MIN_BLOCKS
-#define LBM_FX_MIN_BLOCKS 3
+// Plain steps run in blocks of 128 threads, 6 per SM (80 registers).  The
+// reducing kernel, which runs once per lbm_step call, takes blocks of 256
+// threads (its warp slots are those of lbm_reduce_flux), 3 per SM.
+#ifndef LBM_FX_THREADS
+#define LBM_FX_THREADS 128
 #endif
+#ifndef LBM_FX_MIN_BLOCKS
+#define LBM_FX_MIN_BLOCKS 6
+#endif
+constexpr int kFxThreads = LBM_FX_THREADS;
 #ifndef LBM_FX_RED_MIN_BLOCKS
 #define LBM_FX_RED_MIN_BLOCKS 3
 #endif
@@ -294,18 +295,18 @@ __device__ __forceinline__ bool fx_damp(const int64_t* __restrict__ alpha_fx, in
 }
 
 // A step that does not reduce: n cells, PDF and link rows of stride ld.
-template <int HP_POW2, bool DAMPED>
-__global__ void __launch_bounds__(kSweepThreads, LBM_FX_MIN_BLOCKS)
-    sweep_fx_kernel(const double* __restrict__ src, double* __restrict__ dst,
-                    const int32_t* __restrict__ adj, int32_t n, int32_t ld, FxCoef k,
+template <int HP_POW2, bool DAMPED, bool SHORT>
+__global__ void __launch_bounds__(kFxThreads, LBM_FX_MIN_BLOCKS)
+    sweep_fx_kernel(const double* __restrict__ src, double* __restrict__ dst, Links links,
+                    int32_t n, int32_t ld, FxCoef k,
                     Coef<double> kd, const double* __restrict__ alpha,
                     const int64_t* __restrict__ alpha_fx) {
-  const int32_t i = blockIdx.x * kSweepThreads + threadIdx.x;
+  const int32_t i = blockIdx.x * kFxThreads + threadIdx.x;
   prior_step_done();  // a chained launch waits here for the previous step
+  int32_t idx[18];
+  load_links<SHORT>(links, n, ld, i, idx);
   if (i < n) {
-    int32_t idx[18];
     int64_t b[19];
-    load_links(adj, ld, i, idx);
     fx_pull(src, idx, i, b);
     int64_t S[9], D[9], drho = 0, ux = 0, uy = 0, uz = 0, a1 = 0;
     if (fx_moments(b, k, S, D, drho, ux, uy, uz) &&
@@ -325,10 +326,10 @@ __global__ void __launch_bounds__(kSweepThreads, LBM_FX_MIN_BLOCKS)
 // rather than keep the raw bits live: the reduction then adds little to the
 // registers the collision needs.  (Sharing this structure with the plain
 // step made that one spill.)
-template <int HP_POW2, bool DAMPED>
+template <int HP_POW2, bool DAMPED, bool SHORT>
 __global__ void __launch_bounds__(kSweepThreads, LBM_FX_RED_MIN_BLOCKS)
-    sweep_fx_reduce_kernel(const double* __restrict__ src, double* __restrict__ dst,
-                           const int32_t* __restrict__ adj, int32_t n, int32_t ld, FxCoef k,
+    sweep_fx_reduce_kernel(const double* __restrict__ src, double* __restrict__ dst, Links links,
+                           int32_t n, int32_t ld, FxCoef k,
                            Coef<double> kd, const double* __restrict__ alpha,
                            const int64_t* __restrict__ alpha_fx, double* __restrict__ partials) {
   const int32_t i = blockIdx.x * kSweepThreads + threadIdx.x;
@@ -336,10 +337,10 @@ __global__ void __launch_bounds__(kSweepThreads, LBM_FX_RED_MIN_BLOCKS)
   bool fast = false;
   int64_t S[9], D[9], drho = 0, ux = 0, uy = 0, uz = 0, a1 = 0;
   const int32_t z = prior_step_done();  // zero, after the previous step has finished
+  int32_t idx[18];
+  load_links<SHORT>(links, n, ld, i, idx);
   if (live) {
-    int32_t idx[18];
     int64_t b[19];
-    load_links(adj, ld, i, idx);
     fx_pull(src, idx, i, b);
     fast = fx_moments(b, k, S, D, drho, ux, uy, uz) &&
            fx_damp<DAMPED>(alpha_fx, n, i, k, ux, uy, uz, a1);
@@ -354,7 +355,7 @@ __global__ void __launch_bounds__(kSweepThreads, LBM_FX_RED_MIN_BLOCKS)
       double g[19];
       g[0] = ld_nc(src + i);
 #pragma unroll
-      for (int q = 1; q < 19; ++q) g[q] = ld_nc(src + __ldg(adj + (q - 1) * ld + i));
+      for (int q = 1; q < 19; ++q) g[q] = ld_nc(src + one_link<SHORT>(links, ld, i, q));
       fx_ieee_collide_store<DAMPED>(g, kd, DAMPED ? ld_nc(alpha + i) : 0.0, dst, ld, i, red);
     }
   }
@@ -395,23 +396,39 @@ FxCoef make_fx_coef(double wp, double wm, const double F[3], bool* pow2) {
 // One fixed-point step of state st (its damping included) from src to dst,
 // arrays of rows of stride ld read through links adj; partials non-null: the
 // reducing variant.
-cudaError_t launch_fx(const lbm_state* st, const double* src, double* dst, const int32_t* adj,
-                      int32_t ld, const FxCoef& k, bool pow2, const Coef<double>& kd,
-                      cudaStream_t stream, bool chained, double* partials) {
+template <int P2, bool DA, bool SHORT>
+cudaError_t launch_fx_form(const lbm_state* st, const double* src, double* dst,
+                           const Links& links, int32_t ld, const FxCoef& k,
+                           const Coef<double>& kd, cudaStream_t stream, bool chained,
+                           double* partials) {
   const int32_t n = (int32_t)st->sp->n;
-  const unsigned grid = (unsigned)st->nblocks;
   const double* alpha = (const double*)st->alpha;
   const int64_t* afx = st->alpha_fx;
-#define LBM_FX_LAUNCH(P2, DA)                                                                       \
-  return partials ? launch_sweep(sweep_fx_reduce_kernel<P2, DA>, grid, stream, chained, src, dst, adj, n, ld, k, kd, alpha, afx, partials) \
-                  : launch_sweep(sweep_fx_kernel<P2, DA>, grid, stream, chained, src, dst, adj, n, ld, k, kd, alpha, afx)
-  if (alpha) {
-    if (pow2) { if (k.hp_sign > 0) LBM_FX_LAUNCH(1, true); LBM_FX_LAUNCH(-1, true); }
-    LBM_FX_LAUNCH(0, true);
+  if (partials)
+    return launch_sweep(sweep_fx_reduce_kernel<P2, DA, SHORT>, (unsigned)st->nblocks, stream,
+                        chained, src, dst, links, n, ld, k, kd, alpha, afx, partials);
+  return launch_chained(sweep_fx_kernel<P2, DA, SHORT>, (unsigned)((n + kFxThreads - 1) / kFxThreads),
+                        (unsigned)kFxThreads, stream, chained, src, dst, links, n, ld, k, kd, alpha,
+                        afx);
+}
+cudaError_t launch_fx(const lbm_state* st, const double* src, double* dst, const Links& links,
+                      int32_t ld, const FxCoef& k, bool pow2, const Coef<double>& kd,
+                      cudaStream_t stream, bool chained, double* partials) {
+  const int p2 = !pow2 ? 0 : k.hp_sign;
+#define LBM_FX_FORM(P2, DA)                                                                  \
+  return links.wide ? launch_fx_form<P2, DA, false>(st, src, dst, links, ld, k, kd, stream,  \
+                                                    chained, partials)                       \
+                    : launch_fx_form<P2, DA, true>(st, src, dst, links, ld, k, kd, stream,   \
+                                                   chained, partials)
+  if (st->alpha) {
+    if (p2 > 0) LBM_FX_FORM(1, true);
+    if (p2 < 0) LBM_FX_FORM(-1, true);
+    LBM_FX_FORM(0, true);
   }
-  if (pow2) { if (k.hp_sign > 0) LBM_FX_LAUNCH(1, false); LBM_FX_LAUNCH(-1, false); }
-  LBM_FX_LAUNCH(0, false);
-#undef LBM_FX_LAUNCH
+  if (p2 > 0) LBM_FX_FORM(1, false);
+  if (p2 < 0) LBM_FX_FORM(-1, false);
+  LBM_FX_FORM(0, false);
+#undef LBM_FX_FORM
 }
 
 }  // namespace
@@ -421,12 +438,13 @@ int launch_steps_fx(lbm_state* st, int32_t n_steps, double wp, double wm, const 
   bool pow2 = false;
   const FxCoef k = make_fx_coef(wp, wm, F, &pow2);
   const Coef<double> kd = make_coef<double>(wp, wm, F, 0);
+  const Links links = state_links(st->sp);
   for (int32_t t = 0; t < n_steps; ++t) {
     const double* src = (const double*)st->buf[st->cur];
     double* dst = (double*)st->buf[st->cur ^ 1];
     if (st->sp->n > 0) {
       const bool last = reduce_last && t == n_steps - 1;
-      LBM_CUDA_TRY(launch_fx(st, src, dst, state_links(st->sp), (int32_t)st->sp->ld, k, pow2, kd,
+      LBM_CUDA_TRY(launch_fx(st, src, dst, links, (int32_t)st->sp->ld, k, pow2, kd,
                              stream, t > 0, last ? st->partials : nullptr));
     }
     st->cur ^= 1;
@@ -441,7 +459,8 @@ int launch_fx_step(const lbm_state* st, const double* src, double* dst, const in
   bool pow2 = false;
   const FxCoef k = make_fx_coef(wp, wm, F, &pow2);
   const Coef<double> kd = make_coef<double>(wp, wm, F, 0);
-  LBM_CUDA_TRY(launch_fx(st, src, dst, adj, ld, k, pow2, kd, stream, chained, nullptr));
+  LBM_CUDA_TRY(launch_fx(st, src, dst, Links{adj, nullptr, nullptr}, ld, k, pow2, kd, stream, chained,
+                         nullptr));
   return LBM_OK;
 }
 
