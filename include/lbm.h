@@ -140,8 +140,8 @@ int lbm_ordering_keys(const int32_t dims[3], lbm_ordering ord, uint64_t* keys_de
  *            r*L + m, as int32 (18 rows of L, 72 bytes per L) or, for larger lists
  *            (more than 311,296 cells on GB300), in 16 bits per link and a table of neighbourhoods per 64 cells (38
  *            bytes per L).  adj[18*N] of the layout above is derived from it
- *            on its first request (lbm_sparse_info, lbm_adjoint_create,
- *            lbm_state_create_batched) and then kept; with int32 links and
+ *            on its first request (lbm_sparse_info, lbm_state_create_batched)
+ *            and then kept; with int32 links and
  *            L = N it is the same array.
  * The call synchronises `stream` (to learn N, and again before returning,
  * so the flags may be released afterwards).  Errors: LBM_EINVAL,
@@ -414,10 +414,12 @@ int lbm_halo_gather(const void* src_dev, const int64_t* slots_dev, int64_t count
  * collision of step K, with respect to the body force F and the per-cell
  * Brinkman damping alpha_n, for K steps started from a state's current
  * PDFs: lam_g_K = dJ/dg_K; lam_f_{t-1} = S^T lam_g_t (transposed pull);
- * lam_g_t = C'(g_t)^T lam_f_t (transposed TRT Jacobian).  The forward
- * states are kept as checkpoints every `stride` steps in the state's
- * storage form and recomputed between checkpoints (memory ~ (K/stride +
- * stride) states).  Adjoint arithmetic runs in the state's arithmetic
+ * lam_g_t = C'(g_t)^T lam_f_t (transposed TRT Jacobian).  The reverse
+ * steps need the velocity of each forward step's collision (3 values per
+ * cell).  Within the memory of K/stride + stride states in the state's
+ * storage form, the velocities of as many last steps as fit are kept, and
+ * for the steps before them a few checkpoints, from which they are
+ * recomputed.  Adjoint arithmetic runs in the state's arithmetic
  * precision: FP64 for LBM_F64; for LBM_F64X fixed-point forward steps and
  * double-single reverse steps (lambda as pairs of FP32 values, ~48
  * significant bits, results within 1e-10 of FP64); FP32 otherwise.  Sums in
@@ -426,23 +428,23 @@ int lbm_halo_gather(const void* src_dev, const int64_t* slots_dev, int64_t count
 typedef struct lbm_adjoint lbm_adjoint;
 
 /* Buffers for K = n_steps >= 1 steps of state st (its lattice, form and
- * damping); stride = 0 picks ceil(sqrt(K)).  The adjoint's arrays are
- * [19][N] and read the lattice's public adj[18*N], which this call builds
- * if it is not yet built (see lbm_sparse_info).  The state must outlive
- * every forward and backward pass; lbm_free may release the two in either
- * order. */
+ * damping), at most K/stride + stride + 2 states and two adjoint fields;
+ * stride = 0 picks ceil(sqrt(K)).  Results do not depend on it.  The state
+ * must outlive every forward and backward pass; lbm_free may release the
+ * two in either order. */
 int lbm_adjoint_create(const lbm_state* st, int32_t n_steps, int32_t stride, lbm_adjoint** out);
 
 /* Forward pass from the state's current PDFs (the state is not modified):
- * stores the checkpoints and returns J (axis in {0,1,2}).  Synchronises. */
+ * stores velocities and checkpoints and returns J (axis in {0,1,2}).
+ * Synchronises. */
 int lbm_adjoint_forward(lbm_adjoint* adj, double omega_plus, double omega_minus,
                         const double force[3], int32_t axis, double* J_out);
 
 /* Reverse pass of the last lbm_adjoint_forward.  dJdF_out: host double[3].
  * dJdalpha_dev: device FP64[N] (fluid order), written, or NULL.
  * dJdf0_dev: device FP64[19*N], gradient with respect to the initial PDFs,
- * written, or NULL.  May be called again (it recomputes from the
- * checkpoints).  Synchronises. */
+ * written, or NULL.  May be called again (it recomputes what the first
+ * call overwrote).  Synchronises. */
 int lbm_adjoint_backward(lbm_adjoint* adj, double dJdF_out[3], double* dJdalpha_dev,
                          double* dJdf0_dev);
 

@@ -8,13 +8,6 @@
 //   lam_g_t = C'(g_t)^T lam_f_t  (t = K-1 .. 1),
 // with dJ/dF and dJ/dalpha accumulated from every step.
 //
-// S^T needs no second index array: slot (q, m) is read in the forward pull
-// either by the downstream cell k = m + c_q in direction q, whose
-// adj[q-1][k] = q N + m, or -- when m + c_q is solid or beyond a closed
-// face -- by m itself in direction opp(q) (bounce back).  Both cases are
-// visible in adj[opp(q)-1][m], the pull of direction opp(q) at m, whose
-// source is exactly m + c_q.
-//
 // C'^T is applied in closed form.  Writing the collision as
 //   f*_q = L(g)_q + E_q(rho, u) + S_q(u),
 //   L(g)_q = (1 - (w+ + w-)/2) g_q + ((w- - w+)/2) g_opp(q),
@@ -27,21 +20,51 @@
 //   dJ/dalpha += -(s/2) G.u - 3 (1 - w-/2) M1.u,
 // where M0 = sum w_q lam_q, M1 = sum w_q lam_q c_q, M2 = sum w_q lam_q c_q c_q^T.
 //
-// Memory: checkpoints of f every `stride` steps (stride ~ sqrt(K)) in the
-// state's storage form, one segment of `stride` recomputed states, two
-// adjoint buffers in the arithmetic precision.
+// The reverse step needs g_t only through the velocity u of its collision,
+// three values a cell in place of 19 pulled ones.  So a forward step keeps u
+// (3 rows) rather than f (19 rows): within the memory of a checkpoint every
+// `stride` steps and one segment of `stride` states (stride ~ sqrt(K), as
+// lbm_adjoint_create is asked), U velocity fields cover the last U steps
+// outright, and a few checkpoints of f the rest, recomputed in segments of at
+// most U steps.  Up to K ~ 160 nothing is recomputed in FP32.
+//
+// lambda is kept with its rows reversed: row r holds the adjoint of direction
+// opp(r).  The reader of slot (q, m) is m + c_q, the upwind neighbour of m in
+// direction opp(q), or m itself bounced back -- what the links of direction
+// opp(q) name in row opp(q).  With that, S^T is the pull S itself, through the
+// same links.
+//
+// The reverse steps are bound by bytes: 222 per cell in FP32 (38 links, 12 u,
+// 76 + 76 lambda, 16 dJ/dalpha, 4 alpha; none of the 16 where dJ/dalpha is not
+// asked for) against 320 with g_t pulled from 19 rows through 32-bit links,
+// FP64 storage 398 against 560.  Damped 128^3 bed (1.03 M cells), against that
+// version: 200 steps and their gradient 26.6 -> 17.3 ms in FP32 shifted;
+// reverse pass of 2000 steps (a quarter of them kept) 178 -> 133 ms in FP32
+// shifted, 373 -> 302 in FP64 storage, 1,294 -> 1,031 in IEEE FP64, which is
+// bound by its arithmetic and no longer forms u a second time.
+#include <algorithm>
 #include <cmath>
+#include <type_traits>
 
+#include "double_single.cuh"
 #include "lbm_kernels.cuh"
 
 struct lbm_adjoint {
   uint32_t magic;
   const lbm_state* st;
   cudaStream_t stream;   // the state's stream, kept so that freeing needs no state
-  int32_t K, stride, n_ckpt;
-  void* ckpt;       // n_ckpt states of 19 N storage elements
-  void* seg;        // max(stride, 2) states
-  void* lam[2];     // 19 N arithmetic-precision adjoints
+  int32_t K;
+  // Steps 1..M (M = K - 1) advance f.  u holds the velocities of the last
+  // min(M, slots) steps after a forward pass; the steps before them form n_seg
+  // segments of seg_len steps (the last one may be shorter), each with a
+  // checkpoint of the f it starts from.
+  int32_t slots, n_seg, seg_len;
+  void* ckpt;       // n_seg states of 19 rows of ld storage elements
+  void* f[2];       // the two states steps alternate between
+  void* u;          // slots fields of 3 rows of ld, in the arithmetic precision
+  const void* last; // f_M
+  void* lam[2];     // 19 rows of ld arithmetic-precision adjoints
+  bool fresh;       // lam[0], part, dalpha, u and last are as the forward pass left them
   double* part;     // [nblocks][4]: dJ/dF_x, dJ/dF_y, dJ/dF_z, sum u_axis
   double* dalpha;   // [N]
   double* red_dev;  // [4]
@@ -88,13 +111,6 @@ AdjCoef<C> make_adj_coef(double wp, double wm, int64_t n) {
   a.src12 = (C)((1.0 - 0.5 * wm) / 12.0);
   a.inv_n = (C)(n > 0 ? 1.0 / (double)n : 0.0);
   return a;
-}
-
-// Flat slot, in the adjoint of the pulled values, that holds the adjoint of
-// stored slot (q, i): s = adj[opp(q)-1][i].
-__device__ __forceinline__ int32_t reverse_slot(int q, int32_t s, int32_t n, int32_t i) {
-  const int o = opp(q);
-  return s == q * n + i ? o * n + i : s + (q - o) * n;
 }
 
 // Velocity of the collision of the pulled values g (same arithmetic as the
@@ -144,12 +160,12 @@ __device__ __forceinline__ void block_accumulate4(T v[4], double* acc, bool assi
 }
 
 // Seed: lam_g_K = dJ/dg_K from f_{K-1}; initialises dJ/dF, dJ/dalpha and
-// the sum of u_axis (J = sum / N).
-template <int PREC, bool DAMPED>
+// the sum of u_axis (J = sum / N).  Cells, PDFs, lambda: rows of ld.
+template <int PREC, bool DAMPED, bool SHORT>
 __global__ void __launch_bounds__(kSweepThreads)
-    adjoint_seed_kernel(const typename Form<PREC>::S* __restrict__ f_prev,
-                        const int32_t* __restrict__ adj, int32_t n,
-                        Coef<typename Form<PREC>::C> k, AdjCoef<typename Form<PREC>::C> a,
+    adjoint_seed_kernel(const typename Form<PREC>::S* __restrict__ f_prev, Links links, int32_t n,
+                        int32_t ld, Coef<typename Form<PREC>::C> k,
+                        AdjCoef<typename Form<PREC>::C> a,
                         const typename Form<PREC>::C* __restrict__ alpha, int axis,
                         typename Form<PREC>::C* __restrict__ lam_out, double* __restrict__ part,
                         double* __restrict__ dalpha) {
@@ -159,15 +175,17 @@ __global__ void __launch_bounds__(kSweepThreads)
   const int32_t z = prior_step_done();
   const int32_t i = blockIdx.x * kSweepThreads + threadIdx.x + z;
   double red[4] = {0.0, 0.0, 0.0, 0.0};
+  int32_t idx[18];
+  load_links<SHORT>(links, n, ld, i, idx);
   if (i < n) {
     C g[19];
-    gather<PREC>(f_prev, adj, n, i, k.inv_scale, g);
+    pull<PREC>(f_prev, idx, i, k.inv_scale, g);
     C u[3], s;
     const C al = DAMPED ? alpha[i] : C(0);
     velocity<C, DAMPED>(g, k, al, u, s);
     const C seed = s * a.inv_n;
 #pragma unroll
-    for (int q = 0; q < 19; ++q) lam_out[q * n + i] = C(axis_component(q, axis)) * seed;
+    for (int q = 0; q < 19; ++q) lam_out[opp(q) * ld + i] = C(axis_component(q, axis)) * seed;
     red[axis] = 0.5 * (double)seed;
     red[3] = (double)u[axis];
     dalpha[i] = -0.5 * (double)seed * (double)u[axis];
@@ -175,36 +193,47 @@ __global__ void __launch_bounds__(kSweepThreads)
   block_accumulate4(red, part + z + 4 * (int64_t)blockIdx.x, true);
 }
 
-// One reverse step t: lam_f_t = S^T lam_g_{t+1} (gathered), then
-// lam_g_t = C'(g_t)^T lam_f_t with g_t pulled from f_{t-1}.
-template <int PREC, bool DAMPED>
-__global__ void __launch_bounds__(kSweepThreads)
-    adjoint_step_kernel(const typename Form<PREC>::S* __restrict__ f_prev,
-                        const int32_t* __restrict__ adj, int32_t n,
-                        Coef<typename Form<PREC>::C> k, AdjCoef<typename Form<PREC>::C> a,
-                        const typename Form<PREC>::C* __restrict__ alpha,
-                        const typename Form<PREC>::C* __restrict__ lam_in,
-                        typename Form<PREC>::C* __restrict__ lam_out, double* __restrict__ part,
+__device__ __forceinline__ float2 ld_nc(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.nc" LBM_LD_HINT ".v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+
+// The 19 pulled adjoints of cell i, lf[q] that of direction q.
+template <class T>
+__device__ __forceinline__ void pull_adjoint(const T* __restrict__ lam_in, const int32_t idx[18],
+                                             int32_t i, T lf[19]) {
+  lf[0] = ld_nc(lam_in + i);
+#pragma unroll
+  for (int q = 1; q < 19; ++q) lf[opp(q)] = ld_nc(lam_in + idx[q - 1]);
+}
+
+// One reverse step t: lam_f_t = S^T lam_g_{t+1} (pulled), then
+// lam_g_t = C'(g_t)^T lam_f_t with the velocity u of that collision, rows of
+// ld.  dalpha may be null (dJ/dalpha not wanted).
+// FP32 at 5 resident blocks (48 registers): 200 steps and their gradient on the
+// damped 128^3 bed 17.3 ms, 17.8 at 4 and 17.7 at 6.
+#ifndef LBM_ADJ_MIN_BLOCKS
+#define LBM_ADJ_MIN_BLOCKS 5
+#endif
+template <class C, bool DAMPED, bool SHORT>
+__global__ void __launch_bounds__(kSweepThreads, sizeof(C) == 4 ? LBM_ADJ_MIN_BLOCKS : 1)
+    adjoint_step_kernel(const C* __restrict__ u_in, Links links, int32_t n, int32_t ld,
+                        AdjCoef<C> a, const C* __restrict__ alpha, const C* __restrict__ lam_in,
+                        C* __restrict__ lam_out, double* __restrict__ part,
                         double* __restrict__ dalpha) {
-  using C = typename Form<PREC>::C;
   const int32_t z = prior_step_done();  // as in adjoint_seed_kernel
   const int32_t i = blockIdx.x * kSweepThreads + threadIdx.x + z;
   C red[4] = {C(0), C(0), C(0), C(0)};
+  int32_t idx[18];
+  load_links<SHORT>(links, n, ld, i, idx);
   if (i < n) {
-    int32_t idx[18];
+    C lf[19], u[3];
+    pull_adjoint(lam_in, idx, i, lf);
 #pragma unroll
-    for (int q = 0; q < 18; ++q) idx[q] = __ldg(adj + q * n + i);
-    // all 36 pulls of the cell are independent: issue them back to back
-    C lf[19], g[19];
-    lf[0] = lam_in[i];
-    g[0] = decode<PREC>(load_ro<PREC>(f_prev + i), k.inv_scale);
-#pragma unroll
-    for (int q = 1; q < 19; ++q) g[q] = decode<PREC>(load_ro<PREC>(f_prev + idx[q - 1]), k.inv_scale);
-#pragma unroll
-    for (int q = 1; q < 19; ++q) lf[q] = __ldg(lam_in + reverse_slot(q, idx[opp(q) - 1], n, i));
-    C u[3], s;
-    const C al = DAMPED ? alpha[i] : C(0);
-    velocity<C, DAMPED>(g, k, al, u, s);
+    for (int j = 0; j < 3; ++j) u[j] = ld_nc(u_in + j * ld + i);
+    const C al = DAMPED ? ld_nc(alpha + i) : C(0);
+    const C s = DAMPED ? C(1) / (C(1) + C(0.5) * al) : C(1);
     C S[9], D[9];
 #pragma unroll
     for (int p = 0; p < 9; ++p) {
@@ -243,8 +272,8 @@ __global__ void __launch_bounds__(kSweepThreads)
   {                                                                            \
     const C e_ = a.hp * S[P] + base;                                           \
     const C o_ = a.hm * D[P] + s * (CG);                                       \
-    lam_out[(2 * P + 1) * n + i] = e_ + o_;                                    \
-    lam_out[(2 * P + 2) * n + i] = e_ - o_;                                    \
+    lam_out[(2 * P + 2) * ld + i] = e_ + o_;                                    \
+    lam_out[(2 * P + 1) * ld + i] = e_ - o_;                                    \
   }
       LBM_ADJ_PAIR(0, Gx)
       LBM_ADJ_PAIR(1, Gy)
@@ -263,7 +292,7 @@ __global__ void __launch_bounds__(kSweepThreads)
       red[2] = hs * Gz + a.src12 * M1z;
       const C Gu = Gx * u[0] + Gy * u[1] + Gz * u[2];
       const C M1u = M1x * u[0] + M1y * u[1] + M1z * u[2];
-      dalpha[i] += (double)(-hs * Gu - a.src12 * M1u);
+      if (dalpha) dalpha[i] += (double)(-hs * Gu - a.src12 * M1u);
     } else {
       // weighted moments of the adjoint
       const C w0 = C(1.0 / 3.0), w1 = C(1.0 / 18.0), w2 = C(1.0 / 36.0);
@@ -280,16 +309,22 @@ __global__ void __launch_bounds__(kSweepThreads)
       const C Myz = w2 * (S[7] - S[8]);
       const C nine_wp = C(9) * a.wp, three_wp_m0 = C(3) * a.wp * M0;
       const C beta = C(3) * (a.wm - al * a.src);
-      const C Gx = nine_wp * (Mxx * u[0] + Mxy * u[1] + Mxz * u[2]) - three_wp_m0 * u[0] + beta * M1x;
-      const C Gy = nine_wp * (Mxy * u[0] + Myy * u[1] + Myz * u[2]) - three_wp_m0 * u[1] + beta * M1y;
-      const C Gz = nine_wp * (Mxz * u[0] + Myz * u[1] + Mzz * u[2]) - three_wp_m0 * u[2] + beta * M1z;
+      // G = nine_wp (M2 u) - three_wp_m0 u + beta M1, each rounding written out:
+      // left to the compiler, the sums contract differently from one
+      // instantiation of this kernel to the next
+      const auto G = [&](C q, C uj, C m1) {
+        return __fmaf_rn(beta, m1, __fmaf_rn(nine_wp, q, -__fmul_rn(three_wp_m0, uj)));
+      };
+      const C Gx = G(__fmaf_rn(Mxz, u[2], __fmaf_rn(Mxx, u[0], __fmul_rn(Mxy, u[1]))), u[0], M1x);
+      const C Gy = G(__fmaf_rn(Myz, u[2], __fmaf_rn(Myy, u[1], __fmul_rn(Mxy, u[0]))), u[1], M1y);
+      const C Gz = G(__fmaf_rn(Mzz, u[2], __fmaf_rn(Mxz, u[0], __fmul_rn(Myz, u[1]))), u[2], M1z);
       const C base = a.wp * M0;
       lam_out[i] = a.one_m_wp * lf[0] + base;
 #define LBM_ADJ_PAIR(P, CG)                                                    \
   {                                                                            \
     const C sg_ = s * (CG);                                                    \
-    lam_out[(2 * P + 1) * n + i] = a.k1 * lf[2 * P + 1] + a.k2 * lf[2 * P + 2] + base + sg_; \
-    lam_out[(2 * P + 2) * n + i] = a.k1 * lf[2 * P + 2] + a.k2 * lf[2 * P + 1] + base - sg_; \
+    lam_out[(2 * P + 2) * ld + i] = a.k1 * lf[2 * P + 1] + a.k2 * lf[2 * P + 2] + base + sg_; \
+    lam_out[(2 * P + 1) * ld + i] = a.k1 * lf[2 * P + 2] + a.k2 * lf[2 * P + 1] + base - sg_; \
   }
       LBM_ADJ_PAIR(0, Gx)
       LBM_ADJ_PAIR(1, Gy)
@@ -307,7 +342,7 @@ __global__ void __launch_bounds__(kSweepThreads)
       red[2] = hs * Gz + three_src * M1z;
       const C Gu = Gx * u[0] + Gy * u[1] + Gz * u[2];
       const C M1u = M1x * u[0] + M1y * u[1] + M1z * u[2];
-      dalpha[i] += (double)(-hs * Gu - three_src * M1u);
+      if (dalpha) dalpha[i] += (double)(-hs * Gu - three_src * M1u);
     }
   }
   block_accumulate4(red, part + z + 4 * (int64_t)blockIdx.x, false);
@@ -316,66 +351,15 @@ __global__ void __launch_bounds__(kSweepThreads)
 // ---- FP64-storage adjoint in double-single arithmetic --------------------------
 // For LBM_F64X the reverse step keeps FP64-level accuracy without FP64
 // instructions on its common path.  lambda is stored as a pair of FP32
-// values (hi, lo) whose unevaluated sum carries ~48 significant bits, and
-// is computed with error-free transformations: Knuth's TwoSum, Dekker's
-// Fast2Sum (|a| >= |b|), and the product of two FP32 values with its exact
-// error from one FMA (Ogita, Rump and Oishi, 2005).  The forward velocity
-// comes exact from the FP64 bit patterns in 64-bit fixed point, as in the
-// fixed-point sweep (units 2^-58), damping included (u - e u); a cell whose
-// PDFs leave their binary ranges computes it in FP64 instead.
-struct ds {
-  float hi, lo;
-};
-
-__device__ __forceinline__ ds ds_two_sum(float a, float b) {
-  const float s = a + b;
-  const float bb = s - a;
-  return {s, (a - (s - bb)) + (b - bb)};
-}
-__device__ __forceinline__ ds ds_fast_two_sum(float a, float b) {
-  const float s = a + b;
-  return {s, b - (s - a)};
-}
-__device__ __forceinline__ ds ds_add(ds x, ds y) {
-  const ds s = ds_two_sum(x.hi, y.hi);
-  return ds_fast_two_sum(s.hi, s.lo + (x.lo + y.lo));
-}
-__device__ __forceinline__ ds ds_neg(ds x) { return {-x.hi, -x.lo}; }
-__device__ __forceinline__ ds ds_sub(ds x, ds y) { return ds_add(x, ds_neg(y)); }
-__device__ __forceinline__ ds ds_mul(ds x, ds y) {
-  const float p = x.hi * y.hi;
-  const float e = fmaf(x.hi, y.hi, -p);
-  return ds_fast_two_sum(p, fmaf(x.hi, y.lo, fmaf(x.lo, y.hi, e)));
-}
-// x times a power of two c (exact, barring overflow and underflow)
-__device__ __forceinline__ ds ds_scale_pow2(ds x, float c) { return {x.hi * c, x.lo * c}; }
-__device__ __forceinline__ double ds_to_double(ds x) { return (double)x.hi + (double)x.lo; }
-// Host and device: the pair nearest to v (|lo| <= ulp(hi)/2).
-__host__ __device__ __forceinline__ ds ds_from_double(double v) {
-  const float hi = (float)v;
-  return {hi, (float)(v - (double)hi)};
-}
-// An int64 value in units 2^-sc (sc = 58 or 63, |v| < 2^62), to ~48 bits.
-// 64-bit integer conversions issue at the FP64 rate on GB300, so v is cut
-// into three 21-bit pieces, each converted exactly as a 32-bit integer, and
-// the pieces are summed as pairs.
-__device__ __forceinline__ ds ds_from_fixed(int64_t v, int sc) {
-  const float a = (float)(int32_t)(v >> 42) * 0x1p42f;                 // exact
-  const float b = (float)(int32_t)((v >> 21) & 0x1FFFFF) * 0x1p21f;    // exact
-  const float c = (float)(int32_t)(v & 0x1FFFFF);                      // exact
-  const ds ab = ds_two_sum(a, b);
-  const ds r = ds_add(ab, ds{c, 0.f});
-  const float scale = sc == 58 ? 0x1p-58f : 0x1p-63f;   // exact: powers of two
-  return {r.hi * scale, r.lo * scale};
-}
-
+// values (hi, lo) whose unevaluated sum carries ~48 significant bits
+// (double_single.cuh).  The forward velocity is the one of the fixed-point
+// sweep (exact in units 2^-58), kept as a pair.
 // Coefficients of the reverse step as pairs (those of AdjCoef).
 struct AdjCoefDS {
   ds one_m_wp, hp, hm, wp36, wp12, wp4, wm12, src12;
-  int64_t fhF[3];   // F/2 in units 2^-58, for the fixed-point velocity
 };
 
-AdjCoefDS make_adj_coef_ds(double wp, double wm, const double F[3]) {
+AdjCoefDS make_adj_coef_ds(double wp, double wm) {
   AdjCoefDS a;
   a.one_m_wp = ds_from_double(1.0 - wp);
   a.hp = ds_from_double(0.5 * (1.0 - wp));
@@ -385,60 +369,7 @@ AdjCoefDS make_adj_coef_ds(double wp, double wm, const double F[3]) {
   a.wp4 = ds_from_double(0.25 * wp);
   a.wm12 = ds_from_double(wm / 12.0);
   a.src12 = ds_from_double((1.0 - 0.5 * wm) / 12.0);
-  for (int d = 0; d < 3; ++d) a.fhF[d] = (int64_t)std::llround(0.5 * F[d] * 0x1p58);
   return a;
-}
-
-constexpr int64_t kAdjW0Bits = 0x3FD5555555555555LL;  // bits of 1/3, 1/18, 1/36
-constexpr int64_t kAdjW1Bits = 0x3FAC71C71C71C71CLL;
-constexpr int64_t kAdjW2Bits = 0x3F9C71C71C71C71CLL;
-
-// Velocity and damping factor s = 1/(1 + alpha/2) of the collision of the
-// pulled FP64 values g, as pairs: from the bit patterns in fixed point where
-// every value lies in its weight's binary range (and alpha in [0, 1/2)),
-// else in FP64.
-template <bool DAMPED>
-__device__ __forceinline__ void ds_velocity(const double g[19], const AdjCoefDS& a,
-                                            const Coef<double>& kd,
-                                            const double* __restrict__ alpha,
-                                            const int64_t* __restrict__ alpha_fx, int32_t n,
-                                            int32_t i, ds u[3], ds& s) {
-  bool fast = true;
-  int64_t X[19];
-#pragma unroll
-  for (int q = 0; q < 19; ++q) {
-    const int64_t b = __double_as_longlong(g[q]);
-    const int64_t wb = q == 0 ? kAdjW0Bits : (q <= 6 ? kAdjW1Bits : kAdjW2Bits);
-    const int sh = q == 0 ? 4 : (q <= 6 ? 1 : 0);
-    fast &= (b >> 52) == (wb >> 52);
-    X[q] = (b - wb) << sh;   // exact deviation in units 2^-58 when in range
-  }
-  int64_t E = 0;
-  if constexpr (DAMPED) {
-    const int64_t A = __ldg(alpha_fx + i);
-    fast &= A >= 0;
-    E = __ldg(alpha_fx + n + i);
-  }
-  if (fast) {
-    int64_t D[9];
-#pragma unroll
-    for (int p = 0; p < 9; ++p) D[p] = X[2 * p + 1] - X[2 * p + 2];
-    int64_t j[3] = {(((D[0] + D[3]) + (D[4] + D[5])) + D[6]) + a.fhF[0],
-                    (((D[1] + D[3]) - (D[4] - D[7])) + D[8]) + a.fhF[1],
-                    (((D[2] + D[5]) - (D[6] - D[7])) - D[8]) + a.fhF[2]};
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      if constexpr (DAMPED) j[d] -= __mul64hi(2 * j[d], E);   // u = j - e j
-      u[d] = ds_from_fixed(j[d], 58);
-    }
-    s = DAMPED ? ds_sub(ds{1.f, 0.f}, ds_from_fixed(E, 63)) : ds{1.f, 0.f};
-  } else {
-    double ud[3], sd;
-    velocity<double, DAMPED>(g, kd, DAMPED ? alpha[i] : 0.0, ud, sd);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) u[d] = ds_from_double(ud[d]);
-    s = ds_from_double(sd);
-  }
 }
 
 // Block sums of four pairs, added to acc[4] in FP64 (as block_accumulate4).
@@ -466,18 +397,21 @@ __device__ __forceinline__ void block_accumulate4_ds(ds v[4], double* acc, bool 
 }
 
 // Seed of the FP64-storage adjoint: as adjoint_seed_kernel, lambda written
-// as pairs (float2 [19][N]).
-template <bool DAMPED>
+// as pairs (float2, 19 rows of ld).
+template <bool DAMPED, bool SHORT>
 __global__ void __launch_bounds__(kSweepThreads)
-    adjoint_seed_ds_kernel(const double* __restrict__ f_prev, const int32_t* __restrict__ adj,
-                           int32_t n, Coef<double> k, AdjCoef<double> a,
-                           const double* __restrict__ alpha, int axis, float2* __restrict__ lam_out,
-                           double* __restrict__ part, double* __restrict__ dalpha) {
-  const int32_t i = blockIdx.x * kSweepThreads + threadIdx.x;
+    adjoint_seed_ds_kernel(const double* __restrict__ f_prev, Links links, int32_t n, int32_t ld,
+                           Coef<double> k, AdjCoef<double> a, const double* __restrict__ alpha,
+                           int axis, float2* __restrict__ lam_out, double* __restrict__ part,
+                           double* __restrict__ dalpha) {
+  const int32_t z = prior_step_done();  // as in adjoint_seed_kernel
+  const int32_t i = blockIdx.x * kSweepThreads + threadIdx.x + z;
   double red[4] = {0.0, 0.0, 0.0, 0.0};
+  int32_t idx[18];
+  load_links<SHORT>(links, n, ld, i, idx);
   if (i < n) {
     double g[19];
-    gather<LBM_F64>(f_prev, adj, n, i, 1.0, g);
+    pull<LBM_F64>(f_prev, idx, i, 1.0, g);
     double u[3], s;
     const double al = DAMPED ? alpha[i] : 0.0;
     velocity<double, DAMPED>(g, k, al, u, s);
@@ -485,46 +419,56 @@ __global__ void __launch_bounds__(kSweepThreads)
 #pragma unroll
     for (int q = 0; q < 19; ++q) {
       const ds v = ds_from_double((double)axis_component(q, axis) * seed);
-      lam_out[q * n + i] = make_float2(v.hi, v.lo);
+      lam_out[opp(q) * ld + i] = make_float2(v.hi, v.lo);
     }
     red[axis] = 0.5 * seed;
     red[3] = u[axis];
     dalpha[i] = -0.5 * seed * u[axis];
   }
-  block_accumulate4(red, part + 4 * (int64_t)blockIdx.x, true);
+  block_accumulate4(red, part + z + 4 * (int64_t)blockIdx.x, true);
 }
 
 // One reverse step of the FP64-storage adjoint (adjoint_step_kernel's
 // formulas) in double-single arithmetic.
-// 3 resident blocks per SM (80 registers, 36 bytes spilled): the damped
-// 128^3 reverse pass took 0.392 s against 0.426 s at the 102 registers (2
-// blocks) the compiler picks unbounded, two alternating runs each.
+// 3 resident blocks (80 registers): 60 steps and their gradient on a damped
+// 91x83x117 bed 5.12 ms, 5.16 at 4 and 5.95 at 2.
 #ifndef LBM_ADJ_DS_MIN_BLOCKS
 #define LBM_ADJ_DS_MIN_BLOCKS 3
 #endif
-template <bool DAMPED>
+template <bool DAMPED, bool SHORT>
 __global__ void __launch_bounds__(kSweepThreads, LBM_ADJ_DS_MIN_BLOCKS)
-    adjoint_step_ds_kernel(const double* __restrict__ f_prev, const int32_t* __restrict__ adj,
-                           int32_t n, Coef<double> kd, AdjCoefDS a,
-                           const double* __restrict__ alpha, const int64_t* __restrict__ alpha_fx,
+    adjoint_step_ds_kernel(const float2* __restrict__ u_in, Links links, int32_t n, int32_t ld,
+                           AdjCoefDS a, const double* __restrict__ alpha,
+                           const int64_t* __restrict__ alpha_fx,
                            const float2* __restrict__ lam_in, float2* __restrict__ lam_out,
                            double* __restrict__ part, double* __restrict__ dalpha) {
-  const int32_t i = blockIdx.x * kSweepThreads + threadIdx.x;
+  const int32_t z = prior_step_done();  // as in adjoint_seed_kernel
+  const int32_t i = blockIdx.x * kSweepThreads + threadIdx.x + z;
   ds red[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+  int32_t idx[18];
+  load_links<SHORT>(links, n, ld, i, idx);
   if (i < n) {
-    int32_t idx[18];
-#pragma unroll
-    for (int q = 0; q < 18; ++q) idx[q] = __ldg(adj + q * n + i);
-    double g[19];
     float2 l2[19];
-    g[0] = ld_nc(f_prev + i);
+    pull_adjoint(lam_in, idx, i, l2);
+    ds u[3];
 #pragma unroll
-    for (int q = 1; q < 19; ++q) g[q] = ld_nc(f_prev + idx[q - 1]);
-    l2[0] = __ldg(lam_in + i);
-#pragma unroll
-    for (int q = 1; q < 19; ++q) l2[q] = __ldg(lam_in + reverse_slot(q, idx[opp(q) - 1], n, i));
-    ds u[3], s;
-    ds_velocity<DAMPED>(g, a, kd, alpha, alpha_fx, n, i, u, s);
+    for (int j = 0; j < 3; ++j) {
+      const float2 v = ld_nc(u_in + j * ld + i);
+      u[j] = {v.x, v.y};
+    }
+    // s = 1/(1 + alpha/2) = 1 - e, and alpha, from their fixed-point values
+    // where alpha lies in [0, 1/2)
+    ds s = {1.f, 0.f}, al = {0.f, 0.f};
+    if constexpr (DAMPED) {
+      const int64_t A = __ldg(alpha_fx + i);
+      if (A >= 0) {
+        s = ds_sub(s, ds_from_fixed(__ldg(alpha_fx + n + i), 63));
+        al = ds_from_fixed(A, 63);
+      } else {
+        s = ds_from_double(1.0 / (1.0 + 0.5 * alpha[i]));
+        al = ds_from_double(alpha[i]);
+      }
+    }
     ds lf[19];
 #pragma unroll
     for (int q = 0; q < 19; ++q) lf[q] = {l2[q].x, l2[q].y};
@@ -550,13 +494,9 @@ __global__ void __launch_bounds__(kSweepThreads, LBM_ADJ_DS_MIN_BLOCKS)
     const ds Mxz = ds_sub(S[5], S[6]);
     const ds Myz = ds_sub(S[7], S[8]);
     const ds m0 = ds_mul(a.wp12, M0);
-    // beta/36 = w-/12 - alpha src/12; alpha from its fixed-point value
+    // beta/36 = w-/12 - alpha src/12
     ds beta = a.wm12;
-    if constexpr (DAMPED) {
-      const int64_t A = __ldg(alpha_fx + i);
-      const ds al = A >= 0 ? ds_from_fixed(A, 63) : ds_from_double(alpha[i]);
-      beta = ds_sub(beta, ds_mul(a.src12, al));
-    }
+    if constexpr (DAMPED) beta = ds_sub(beta, ds_mul(a.src12, al));
     const ds Gx = ds_add(ds_sub(ds_mul(a.wp4, ds_add(ds_add(ds_mul(Mxx, u[0]), ds_mul(Mxy, u[1])), ds_mul(Mxz, u[2]))),
                                 ds_mul(m0, u[0])), ds_mul(beta, M1x));
     const ds Gy = ds_add(ds_sub(ds_mul(a.wp4, ds_add(ds_add(ds_mul(Mxy, u[0]), ds_mul(Myy, u[1])), ds_mul(Myz, u[2]))),
@@ -574,8 +514,8 @@ __global__ void __launch_bounds__(kSweepThreads, LBM_ADJ_DS_MIN_BLOCKS)
     const ds o_ = ds_add(ds_mul(a.hm, D[P]), ds_mul(s, (CG)));                                  \
     const ds va_ = ds_add(e_, o_);                                                              \
     const ds vb_ = ds_sub(e_, o_);                                                              \
-    lam_out[(2 * P + 1) * n + i] = make_float2(va_.hi, va_.lo);                                \
-    lam_out[(2 * P + 2) * n + i] = make_float2(vb_.hi, vb_.lo);                                \
+    lam_out[(2 * P + 2) * ld + i] = make_float2(va_.hi, va_.lo);                                \
+    lam_out[(2 * P + 1) * ld + i] = make_float2(vb_.hi, vb_.lo);                                \
   }
     LBM_ADJ_DS_PAIR(0, Gx)
     LBM_ADJ_DS_PAIR(1, Gy)
@@ -593,37 +533,27 @@ __global__ void __launch_bounds__(kSweepThreads, LBM_ADJ_DS_MIN_BLOCKS)
     red[2] = ds_add(ds_mul(hs, Gz), ds_mul(a.src12, M1z));
     const ds Gu = ds_add(ds_add(ds_mul(Gx, u[0]), ds_mul(Gy, u[1])), ds_mul(Gz, u[2]));
     const ds M1u = ds_add(ds_add(ds_mul(M1x, u[0]), ds_mul(M1y, u[1])), ds_mul(M1z, u[2]));
-    dalpha[i] += ds_to_double(ds_neg(ds_add(ds_mul(hs, Gu), ds_mul(a.src12, M1u))));
+    if (dalpha) dalpha[i] += ds_to_double(ds_neg(ds_add(ds_mul(hs, Gu), ds_mul(a.src12, M1u))));
   }
-  block_accumulate4_ds(red, part + 4 * (int64_t)blockIdx.x, false);
+  block_accumulate4_ds(red, part + z + 4 * (int64_t)blockIdx.x, false);
 }
 
-// lam_f_0 of the FP64-storage adjoint (lambda as pairs).
+// lam_f_0 = S^T lam_g_1 (gradient with respect to the initial PDFs, [19][n]).
+__device__ __forceinline__ double as_double(double v) { return v; }
+__device__ __forceinline__ double as_double(float v) { return (double)v; }
+__device__ __forceinline__ double as_double(float2 v) { return (double)v.x + (double)v.y; }
+template <class T, bool SHORT>
 __global__ void __launch_bounds__(kSweepThreads)
-    adjoint_initial_ds_kernel(const int32_t* __restrict__ adj, int32_t n,
-                              const float2* __restrict__ lam_in, double* __restrict__ out) {
+    adjoint_initial_kernel(Links links, int32_t n, int32_t ld, const T* __restrict__ lam_in,
+                           double* __restrict__ out) {
   const int32_t i = blockIdx.x * kSweepThreads + threadIdx.x;
+  int32_t idx[18];
+  load_links<SHORT>(links, n, ld, i, idx);
   if (i >= n) return;
-  const float2 v0 = lam_in[i];
-  out[i] = (double)v0.x + (double)v0.y;
+  T lf[19];
+  pull_adjoint(lam_in, idx, i, lf);
 #pragma unroll
-  for (int q = 1; q < 19; ++q) {
-    const float2 v = lam_in[reverse_slot(q, adj[(opp(q) - 1) * n + i], n, i)];
-    out[q * n + i] = (double)v.x + (double)v.y;
-  }
-}
-
-// lam_f_0 = S^T lam_g_1 (gradient with respect to the initial PDFs).
-template <class C>
-__global__ void __launch_bounds__(kSweepThreads)
-    adjoint_initial_kernel(const int32_t* __restrict__ adj, int32_t n,
-                           const C* __restrict__ lam_in, double* __restrict__ out) {
-  const int32_t i = blockIdx.x * kSweepThreads + threadIdx.x;
-  if (i >= n) return;
-  out[i] = (double)lam_in[i];
-#pragma unroll
-  for (int q = 1; q < 19; ++q)
-    out[q * n + i] = (double)lam_in[reverse_slot(q, adj[(opp(q) - 1) * n + i], n, i)];
+  for (int q = 0; q < 19; ++q) out[q * (int64_t)n + i] = as_double(lf[q]);
 }
 
 // ---- host orchestration -------------------------------------------------------
@@ -632,127 +562,143 @@ template <int PREC>
 struct Runner {
   using S = typename Form<PREC>::S;
   using C = typename Form<PREC>::C;
+  // an element of lambda and of the kept velocities
+  using E = std::conditional_t<PREC == LBM_F64X, float2, C>;
   lbm_adjoint* ad;
   const lbm_state* st;
-  int32_t n;
+  int32_t n, ld, M;
   cudaStream_t stream;
   unsigned grid;
+  Links links;
   Coef<C> k;
   AdjCoef<C> a;
-  const C* alpha;
-  size_t state_elems;
+  AdjCoefDS ads;   // LBM_F64X: the reverse step in double-single arithmetic
   // Kernels after the first of a forward or backward pass are chained
   // (programmatic dependent launch; the kernels wait for their predecessor),
   // except in FP64 arithmetic, which chaining slows down.
-  static constexpr bool kChain = PREC != LBM_F64 && PREC != LBM_F64X;
-  mutable bool chained = false;
-  mutable cudaError_t err = cudaSuccess;
+  static constexpr bool kChain = PREC != LBM_F64;
+  bool chained = false;
+  cudaError_t err = cudaSuccess;
 
-  AdjCoefDS ads;   // LBM_F64X: the reverse step in double-single arithmetic
   Runner(lbm_adjoint* ad_) : ad(ad_), st(ad_->st) {
     n = (int32_t)st->sp->n;
+    ld = (int32_t)st->sp->ld;
+    M = ad->K - 1;
     stream = st->sp->stream;
     grid = (unsigned)st->nblocks;
+    links = state_links(st->sp);
     k = make_coef<C>(ad->wp, ad->wm, ad->F, st->scale_exp);
     a = make_adj_coef<C>(ad->wp, ad->wm, n);
-    alpha = (const C*)st->alpha;
-    state_elems = 19 * (size_t)n;
-    if constexpr (PREC == LBM_F64X) ads = make_adj_coef_ds(ad->wp, ad->wm, ad->F);
+    if constexpr (PREC == LBM_F64X) ads = make_adj_coef_ds(ad->wp, ad->wm);
   }
-  float2* lam2(int i) const { return (float2*)ad->lam[i]; }
-  S* ckpt(int j) const { return (S*)ad->ckpt + (size_t)j * state_elems; }
-  S* seg(int i) const { return (S*)ad->seg + (size_t)i * state_elems; }
-  C* lam(int i) const { return (C*)ad->lam[i]; }
+  S* ckpt(int j) const { return (S*)ad->ckpt + (size_t)j * 19 * ld; }
+  E* u(int slot) const { return (E*)ad->u + (size_t)slot * 3 * ld; }
+  E* lam(int i) const { return (E*)ad->lam[i]; }
 
   template <class... P, class... A>
-  void launch(void (*kernel)(P...), A... args) const {
+  void launch(void (*kernel)(P...), A... args) {
     const cudaError_t e = launch_sweep(kernel, grid, stream, kChain && chained, args...);
     if (err == cudaSuccess) err = e;
     chained = true;
   }
-  void step(const S* src, S* dst) const {
-    if constexpr (PREC == LBM_F64X) {
-      // FP64 storage: the fixed-point sweep, as lbm_step takes it
-      const int rc = launch_fx_step(st, (const double*)src, (double*)dst, st->sp->adj, n, ad->wp,
-                                    ad->wm, ad->F, stream, false);
-      if (rc != LBM_OK && err == cudaSuccess) err = cudaErrorLaunchFailure;
-      chained = true;
-      return;
-    }
-    if (alpha) launch(sweep_kernel<PREC, true, kNoReduce>, src, dst, Links{st->sp->adj, nullptr, nullptr}, n, n, k, alpha, (double*)nullptr);
-    else launch(sweep_kernel<PREC, false, kNoReduce>, src, dst, Links{st->sp->adj, nullptr, nullptr}, n, n, k, alpha, (double*)nullptr);
+  void step(const void* src, void* dst, E* u_out) {
+    const cudaError_t e = launch_plain_step(st, src, dst, u_out, ad->wp, ad->wm, ad->F, stream,
+                                            kChain && chained);
+    if (err == cudaSuccess) err = e;
+    chained = true;
   }
-  void seed(const S* f_prev) const {
-    if constexpr (PREC == LBM_F64X) {
-      const double* al = (const double*)alpha;
-      if (alpha) launch(adjoint_seed_ds_kernel<true>, (const double*)f_prev, st->sp->adj, n, k, a, al, ad->axis, lam2(0), ad->part, ad->dalpha);
-      else launch(adjoint_seed_ds_kernel<false>, (const double*)f_prev, st->sp->adj, n, k, a, al, ad->axis, lam2(0), ad->part, ad->dalpha);
-      return;
-    }
-    if (alpha) launch(adjoint_seed_kernel<PREC, true>, f_prev, st->sp->adj, n, k, a, alpha, ad->axis, lam(0), ad->part, ad->dalpha);
-    else launch(adjoint_seed_kernel<PREC, false>, f_prev, st->sp->adj, n, k, a, alpha, ad->axis, lam(0), ad->part, ad->dalpha);
+  template <bool DA, bool SH>
+  void seed_form(const S* f_prev) {
+    const C* alpha = (const C*)st->alpha;
+    if constexpr (PREC == LBM_F64X)
+      launch(adjoint_seed_ds_kernel<DA, SH>, f_prev, links, n, ld, k, a, alpha, ad->axis, lam(0),
+             ad->part, ad->dalpha);
+    else
+      launch(adjoint_seed_kernel<PREC, DA, SH>, f_prev, links, n, ld, k, a, alpha, ad->axis,
+             lam(0), ad->part, ad->dalpha);
   }
-  void reverse(const S* f_prev, int in) const {
-    if constexpr (PREC == LBM_F64X) {
-      const double* al = (const double*)alpha;
-      if (alpha) launch(adjoint_step_ds_kernel<true>, (const double*)f_prev, st->sp->adj, n, k, ads, al, (const int64_t*)st->alpha_fx, (const float2*)lam2(in), lam2(in ^ 1), ad->part, ad->dalpha);
-      else launch(adjoint_step_ds_kernel<false>, (const double*)f_prev, st->sp->adj, n, k, ads, al, (const int64_t*)st->alpha_fx, (const float2*)lam2(in), lam2(in ^ 1), ad->part, ad->dalpha);
-      return;
-    }
-    if (alpha) launch(adjoint_step_kernel<PREC, true>, f_prev, st->sp->adj, n, k, a, alpha, lam(in), lam(in ^ 1), ad->part, ad->dalpha);
-    else launch(adjoint_step_kernel<PREC, false>, f_prev, st->sp->adj, n, k, a, alpha, lam(in), lam(in ^ 1), ad->part, ad->dalpha);
+  void seed() {
+    const S* f_prev = (const S*)ad->last;
+    if (links.wide) st->alpha ? seed_form<true, false>(f_prev) : seed_form<false, false>(f_prev);
+    else st->alpha ? seed_form<true, true>(f_prev) : seed_form<false, true>(f_prev);
+  }
+  template <bool DA, bool SH>
+  void reverse_form(const E* u_in, int in, double* dalpha) {
+    const C* alpha = (const C*)st->alpha;
+    if constexpr (PREC == LBM_F64X)
+      launch(adjoint_step_ds_kernel<DA, SH>, u_in, links, n, ld, ads, alpha,
+             (const int64_t*)st->alpha_fx, (const float2*)lam(in), lam(in ^ 1), ad->part, dalpha);
+    else
+      launch(adjoint_step_kernel<C, DA, SH>, u_in, links, n, ld, a, alpha, (const C*)lam(in),
+             lam(in ^ 1), ad->part, dalpha);
+  }
+  void reverse(const E* u_in, int in, double* dalpha) {
+    if (links.wide)
+      st->alpha ? reverse_form<true, false>(u_in, in, dalpha) : reverse_form<false, false>(u_in, in, dalpha);
+    else
+      st->alpha ? reverse_form<true, true>(u_in, in, dalpha) : reverse_form<false, true>(u_in, in, dalpha);
   }
 
-  // Forward pass from the state's current PDFs: checkpoints f_{j*stride};
-  // *last receives where f_{K-1} is.  The adjoint's arrays are [19][N] and
-  // read through the plain links; the state's rows have stride sp->ld.
-  int forward(const S** last) const {
-    LBM_CUDA_TRY(cudaMemcpy2DAsync(ckpt(0), (size_t)n * sizeof(S), st->buf[st->cur],
-                                   (size_t)st->sp->ld * sizeof(S), (size_t)n * sizeof(S), 19,
-                                   cudaMemcpyDeviceToDevice, stream));
-    chained = false;
-    const S* cur = ckpt(0);
-    for (int32_t t = 1; t <= ad->K - 1; ++t) {
-      S* dst = (t % ad->stride == 0) ? ckpt(t / ad->stride) : seg(t & 1);
-      step(cur, dst);
+  // First step of segment j (j = n_seg: of the last steps, whose velocities
+  // the forward pass keeps).
+  int32_t first(int j) const {
+    return j < ad->n_seg ? j * ad->seg_len + 1 : M - std::min(M, ad->slots) + 1;
+  }
+
+  // Steps t0..t1 from f_{t0-1} = cur, keeping the velocities of those from
+  // `keep` on in slots 0, 1, ...; with `checkpoints`, the f a segment starts
+  // from goes to its checkpoint.  Returns f_{t1}.
+  const void* advance(const void* cur, int32_t t0, int32_t t1, int32_t keep, bool checkpoints) {
+    int j = 1;
+    for (int32_t t = t0; t <= t1; ++t) {
+      while (j < ad->n_seg && first(j) <= t) ++j;
+      void* dst = checkpoints && j < ad->n_seg && first(j) == t + 1 ? (void*)ckpt(j)
+                  : cur == ad->f[0]                                 ? ad->f[1]
+                                                                    : ad->f[0];
+      step(cur, dst, t >= keep ? u(t - keep) : nullptr);
       cur = dst;
     }
-    *last = cur;
+    return cur;
+  }
+
+  // Forward pass from the state's current PDFs.
+  int forward() {
+    const size_t bytes = 19 * (size_t)ld * sizeof(S);
+    const void* cur = st->buf[st->cur];
+    // the PDFs a later reverse pass starts over from
+    void* copy = ad->n_seg > 0 ? ad->ckpt : (M == 0 ? ad->f[0] : nullptr);
+    if (copy) {
+      LBM_CUDA_TRY(cudaMemcpyAsync(copy, cur, bytes, cudaMemcpyDeviceToDevice, stream));
+      cur = copy;
+    }
+    chained = false;
+    ad->last = advance(cur, 1, M, first(ad->n_seg), true);
+    seed();
+    ad->fresh = true;
     return LBM_OK;
   }
 
-  // Recompute segment j: f_{j*stride + i} for i = 0..last into seg slots
-  // (slot 0 is the checkpoint itself).
-  void recompute(int j, int last) const {
-    const S* cur = ckpt(j);
-    for (int i = 1; i <= last; ++i) {
-      step(cur, seg(i));
-      cur = seg(i);
-    }
-  }
-  const S* state_at(int j, int i) const { return i == 0 ? ckpt(j) : seg(i); }
-
-  int backward(double* dJdf0) const {
-    const int K = ad->K, s = ad->stride;
-    int j = (K - 1) / s;
+  int backward(double* dJdf0, double* dalpha) {
+    const int32_t kept = first(ad->n_seg);
     chained = false;
-    recompute(j, (K - 1) - j * s);
-    seed(state_at(j, (K - 1) - j * s));
+    if (!ad->fresh) {   // a second reverse pass: everything the first one overwrote
+      if (ad->n_seg > 0)
+        ad->last = advance(ckpt(ad->n_seg - 1), first(ad->n_seg - 1), M, kept, false);
+      seed();
+    }
+    ad->fresh = false;
     int in = 0;
-    for (int t = K - 1; t >= 1; --t) {
-      const int jj = (t - 1) / s;
-      if (jj != j) {
-        j = jj;
-        recompute(j, s - 1);
-      }
-      reverse(state_at(j, (t - 1) - j * s), in);
-      in ^= 1;
+    for (int32_t t = M; t >= kept; --t, in ^= 1) reverse(u(t - kept), in, dalpha);
+    for (int j = ad->n_seg - 1; j >= 0; --j) {
+      const int32_t t0 = first(j), t1 = first(j + 1) - 1;
+      advance(ckpt(j), t0, t1, t0, false);
+      for (int32_t t = t1; t >= t0; --t, in ^= 1) reverse(u(t - t0), in, dalpha);
     }
     if (dJdf0) {
-      if constexpr (PREC == LBM_F64X)
-        adjoint_initial_ds_kernel<<<grid, kSweepThreads, 0, stream>>>(st->sp->adj, n, lam2(in), dJdf0);
+      if (links.wide)
+        adjoint_initial_kernel<E, false><<<grid, kSweepThreads, 0, stream>>>(links, n, ld, (const E*)lam(in), dJdf0);
       else
-        adjoint_initial_kernel<C><<<grid, kSweepThreads, 0, stream>>>(st->sp->adj, n, lam(in), dJdf0);
+        adjoint_initial_kernel<E, true><<<grid, kSweepThreads, 0, stream>>>(links, n, ld, (const E*)lam(in), dJdf0);
     }
     LBM_CUDA_TRY(err);
     LBM_CUDA_TRY(cudaGetLastError());
@@ -764,20 +710,20 @@ template <int PREC>
 int run_forward(lbm_adjoint* ad) {
   Runner<PREC> r(ad);
   if (r.n == 0) return LBM_OK;
-  const typename Runner<PREC>::S* last = nullptr;
-  const int rc = r.forward(&last);
+  ad->fresh = false;
+  const int rc = r.forward();
   if (rc != LBM_OK) return rc;
-  r.seed(last);
+  if (r.err != cudaSuccess) ad->fresh = false;
   LBM_CUDA_TRY(r.err);
   LBM_CUDA_TRY(cudaGetLastError());
   return LBM_OK;
 }
 
 template <int PREC>
-int run_backward(lbm_adjoint* ad, double* dJdf0) {
+int run_backward(lbm_adjoint* ad, double* dJdf0, double* dalpha) {
   Runner<PREC> r(ad);
   if (r.n == 0) return LBM_OK;
-  return r.backward(dJdf0);
+  return r.backward(dJdf0, dalpha);
 }
 
 #define LBM_ADJ_DISPATCH(prec, fn, ...)                      \
@@ -791,8 +737,8 @@ int run_backward(lbm_adjoint* ad, double* dJdf0) {
   }
 
 int dispatch_forward(lbm_adjoint* ad) { LBM_ADJ_DISPATCH(ad->st->precision, run_forward, ad) }
-int dispatch_backward(lbm_adjoint* ad, double* dJdf0) {
-  LBM_ADJ_DISPATCH(ad->st->precision, run_backward, ad, dJdf0)
+int dispatch_backward(lbm_adjoint* ad, double* dJdf0, double* dalpha) {
+  LBM_ADJ_DISPATCH(ad->st->precision, run_backward, ad, dJdf0, dalpha)
 }
 
 bool valid_adjoint(const lbm_adjoint* ad) { return ad && ad->magic == kMagicAdjoint; }
@@ -819,7 +765,7 @@ void free_adjoint(lbm_adjoint* ad) {
   // in either order): only the stream kept here is used
   const cudaStream_t s = ad->stream;
   cudaStreamSynchronize(s);
-  for (void* p : {ad->ckpt, ad->seg, ad->lam[0], ad->lam[1], (void*)ad->part,
+  for (void* p : {ad->ckpt, ad->f[0], ad->f[1], ad->u, ad->lam[0], ad->lam[1], (void*)ad->part,
                   (void*)ad->dalpha, (void*)ad->red_dev})
     dev_free(p, s, false);
   if (ad->red_host) cudaFreeHost(ad->red_host);
@@ -843,25 +789,36 @@ extern "C" int lbm_adjoint_create(const lbm_state* st, int32_t n_steps, int32_t 
   if (stride < 0) return fail(LBM_EINVAL, "checkpoint stride %d < 0", stride);
   if (stride == 0) stride = (int32_t)std::ceil(std::sqrt((double)n_steps));
   if (stride > n_steps) stride = n_steps;
-  // the adjoint's arrays are [19][N], read through the public links
-  const int rc = public_links(st->sp, nullptr);
-  if (rc != LBM_OK) return rc;
   lbm_adjoint* ad = new lbm_adjoint{};
   ad->magic = kMagicAdjoint;
   ad->st = st;
   ad->stream = st->sp->stream;
   ad->K = n_steps;
-  ad->stride = stride;
-  ad->n_ckpt = (n_steps - 1) / stride + 1;
   const size_t n = (size_t)(st->sp->n > 0 ? st->sp->n : 1);
-  const size_t sbytes = storage_bytes(st->precision) * 19 * n;
-  const size_t cbytes = compute_bytes(st->precision) * 19 * n;
-  const int nseg = stride > 2 ? stride : 2;
+  const size_t ld = (size_t)(st->sp->ld > 0 ? st->sp->ld : 1);
+  const size_t srow = storage_bytes(st->precision) * ld, crow = compute_bytes(st->precision) * ld;
+  // The memory asked for: a checkpoint every `stride` steps and a segment of
+  // `stride` states, in rows.  Two states and n_seg checkpoints leave the rest
+  // to velocities; the fewest segments none of which is longer than those.
+  const int64_t M = n_steps - 1;
+  const int64_t states = M / stride + 1 + std::max(stride, 2);
+  const int64_t per_slot = 3 * (int64_t)(crow / srow);
+  int64_t seg = 0, slots = 0;
+  for (;; ++seg) {
+    slots = std::min(M, (19 * (states - 2 - seg)) / per_slot);
+    if (slots * (seg + 1) >= M) break;
+  }
+  ad->slots = (int32_t)slots;
+  ad->n_seg = (int32_t)seg;
+  ad->seg_len = seg > 0 ? (int32_t)((M - slots + seg - 1) / seg) : 0;
+  if (seg > 0) ad->n_seg = (int32_t)((M - slots + ad->seg_len - 1) / ad->seg_len);
   const cudaStream_t s = st->sp->stream;
-  bool ok = dev_alloc(&ad->ckpt, sbytes * ad->n_ckpt, s, false) == cudaSuccess &&
-            dev_alloc(&ad->seg, sbytes * nseg, s, false) == cudaSuccess &&
-            dev_alloc(&ad->lam[0], cbytes, s, false) == cudaSuccess &&
-            dev_alloc(&ad->lam[1], cbytes, s, false) == cudaSuccess &&
+  const auto rows = [&](void** p, size_t count, size_t row) {
+    return count == 0 || dev_alloc(p, count * row, s, false) == cudaSuccess;
+  };
+  bool ok = rows(&ad->ckpt, 19 * (size_t)ad->n_seg, srow) && rows(&ad->f[0], 19, srow) &&
+            rows(&ad->f[1], M > 1 ? 19 : 0, srow) && rows(&ad->u, 3 * (size_t)ad->slots, crow) &&
+            rows(&ad->lam[0], 19, crow) && rows(&ad->lam[1], 19, crow) &&
             dev_alloc(&ad->part, sizeof(double) * 4 * st->nblocks, s, false) == cudaSuccess &&
             dev_alloc(&ad->dalpha, sizeof(double) * n, s, false) == cudaSuccess &&
             dev_alloc(&ad->red_dev, sizeof(double) * 4, s, false) == cudaSuccess &&
@@ -869,9 +826,11 @@ extern "C" int lbm_adjoint_create(const lbm_state* st, int32_t n_steps, int32_t 
             cudaEventCreateWithFlags(&ad->done, cudaEventDisableTiming) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
+    const int32_t ad_seg = ad->n_seg;
     free_adjoint(ad);
-    return fail(LBM_ENOMEM, "adjoint allocation failed (%d checkpoints + %d segment states of %zu bytes)",
-                (int)((n_steps - 1) / stride + 1), nseg, sbytes);
+    return fail(LBM_ENOMEM,
+                "adjoint allocation failed (%d checkpoints of %zu bytes, %d velocity fields of %zu)",
+                (int)ad_seg, 19 * srow, (int)slots, 3 * crow);
   }
   *out = ad;
   return LBM_OK;
@@ -910,7 +869,7 @@ extern "C" int lbm_adjoint_backward(lbm_adjoint* ad, double dJdF_out[3], double*
   if (!valid_adjoint(ad)) return fail(LBM_EINVAL, "not an adjoint handle");
   if (!valid_state(ad->st)) return fail(LBM_EINVAL, "the adjoint's state was released");
   if (!ad->have_forward) return fail(LBM_EINVAL, "lbm_adjoint_forward has not run");
-  int rc = dispatch_backward(ad, dJdf0_dev);
+  int rc = dispatch_backward(ad, dJdf0_dev, dJdalpha_dev ? ad->dalpha : nullptr);
   if (rc != LBM_OK) return rc;
   const cudaStream_t stream = ad->st->sp->stream;
   const int64_t n = ad->st->sp->n;

@@ -445,17 +445,21 @@ void free_adjoint(lbm_adjoint* ad);
 size_t storage_bytes(int prec);   // bytes per stored PDF of a precision form
 size_t compute_bytes(int prec);   // bytes of the arithmetic type of a form
 bool is_shifted(int prec);        // stores f - w_q rather than f
-// Fixed-point FP64-storage sweep (sweep_fx.cu), undamped: n_steps launches
-// on `stream`; the last one writes the warp sums when reduce_last is set.
-// One fixed-point step of FP64-storage state st (its damping) from src to
-// dst, arrays of rows of stride ld read through links adj (not reducing),
-// queued on `stream`.
-int launch_fx_step(const lbm_state* st, const double* src, double* dst, const int32_t* adj,
-                   int32_t ld, double wp, double wm, const double F[3], cudaStream_t stream,
-                   bool chained);
+// One plain step (not reducing) of state st -- its lattice, form and damping --
+// from src to dst, PDFs in rows of sp->ld, queued on `stream`.  u_out, if not
+// null, receives the velocity of the step's collision, 3 rows of ld: in the
+// arithmetic precision, for LBM_F64X as pairs of FP32 values.
+cudaError_t launch_plain_step(const lbm_state* st, const void* src, void* dst, void* u_out,
+                              double wp, double wm, const double F[3], cudaStream_t stream,
+                              bool chained);
+cudaError_t launch_fx_step(const lbm_state* st, const double* src, double* dst, void* u_out,
+                           double wp, double wm, const double F[3], cudaStream_t stream,
+                           bool chained);
 // Fills the fixed-point damping rows (alpha_fx) of an FP64-storage state
 // from FP64 alpha on the device.
 int set_alpha_fx(lbm_state* st, const double* alpha_dev);
+// Fixed-point FP64-storage steps (sweep_fx.cu): n_steps launches on `stream`;
+// the last one writes the warp sums when reduce_last is set.
 int launch_steps_fx(lbm_state* st, int32_t n_steps, double wp, double wm, const double F[3],
                     cudaStream_t stream, bool reduce_last);
 bool valid_state(const lbm_state* st);

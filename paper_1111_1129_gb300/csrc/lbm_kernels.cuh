@@ -149,6 +149,9 @@ __device__ __forceinline__ void st_cs(double* p, double v) {
 __device__ __forceinline__ void st_cs(float* p, float v) {
   asm volatile("st.global.cs.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
 }
+__device__ __forceinline__ void st_cs_pair(float* p, float a, float b) {   // p 8-byte aligned
+  asm volatile("st.global.cs.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
+}
 __device__ __forceinline__ void st_cs(unsigned short* p, unsigned short v) {
   asm volatile("st.global.cs.u16 [%0], %1;" ::"l"(p), "h"(v) : "memory");
 }
@@ -538,8 +541,9 @@ constexpr int sweep_min_blocks() {
 }
 
 // RED: 0 no reduction; 1 warp sums into per-warp slots (no block barrier);
-// 2 block sums into per-block slots.  Both give the same final sums.
-enum { kNoReduce = 0, kWarpSums = 1, kBlockSums = 2 };
+// 2 block sums into per-block slots, both giving the same final sums;
+// 3 no reduction, the velocity kept in u_out (3 rows of ld) for the adjoint.
+enum { kNoReduce = 0, kWarpSums = 1, kBlockSums = 2, kKeepU = 3 };
 
 // Resident blocks per SM the reducing variants of the FP32 and 16-bit
 // forms are fitted to: 4 keeps them at the plain variant's 64 registers
@@ -551,7 +555,7 @@ enum { kNoReduce = 0, kWarpSums = 1, kBlockSums = 2 };
 
 template <int PREC, int RED>
 constexpr int sweep_launch_min_blocks() {
-  return RED != kNoReduce && PREC != LBM_F64 && PREC != LBM_F64X ? LBM_RED_MIN_BLOCKS
+  return RED != kNoReduce && RED != kKeepU && PREC != LBM_F64 && PREC != LBM_F64X ? LBM_RED_MIN_BLOCKS
                                                                  : sweep_min_blocks<PREC>();
 }
 
@@ -568,7 +572,8 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_launch_min_blocks<PREC, R
     sweep_kernel(const typename Form<PREC>::S* __restrict__ src,
                  typename Form<PREC>::S* __restrict__ dst, Links links,
                  int32_t n, int32_t ld, Coef<typename Form<PREC>::C> k,
-                 const typename Form<PREC>::C* __restrict__ alpha, double* __restrict__ partials) {
+                 const typename Form<PREC>::C* __restrict__ alpha, double* __restrict__ partials,
+                 typename Form<PREC>::C* __restrict__ u_out) {
   using C = typename Form<PREC>::C;
   const int32_t i = blockIdx.x * kSweepThreads + threadIdx.x;
   C rho = C(0), u[3] = {C(0), C(0), C(0)};
@@ -583,8 +588,11 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_launch_min_blocks<PREC, R
     collide<C, DAMPED>(g, k, DAMPED ? ld_nc(alpha + i) : C(0), rho, u);
 #pragma unroll
     for (int q = 0; q < 19; ++q) store_stream<PREC>(dst + q * ld + i, encode<PREC>(g[q], k.scale));
+    if constexpr (RED == kKeepU)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) st_cs(u_out + j * ld + i, u[j]);
   }
-  if constexpr (RED != kNoReduce) {
+  if constexpr (RED == kWarpSums || RED == kBlockSums) {
     double w[4];
     warp_flux_sums<C, Form<PREC>::kShifted>(i < n, rho, u, w);
     if constexpr (RED == kWarpSums) store_warp_sums(w, partials + z);
@@ -654,11 +662,12 @@ __device__ __forceinline__ void load_pair_links(const Links& links, int32_t ld, 
   entry = page_entry(links, i);
 }
 
-template <int PREC, bool DAMPED>
+template <int PREC, bool DAMPED, bool KEEP_U>
 __global__ void __launch_bounds__(kPairThreads, LBM_PAIR_MIN_BLOCKS)
     sweep_pair_kernel(const typename Form<PREC>::S* __restrict__ src,
                       typename Form<PREC>::S* __restrict__ dst, Links links, int32_t n,
-                      int32_t ld, Coef<float> k, const float* __restrict__ alpha) {
+                      int32_t ld, Coef<float> k, const float* __restrict__ alpha,
+                      float* __restrict__ u_out) {
   static_assert(PREC == LBM_F16S || PREC == LBM_BF16S, "16-bit forms only");
   const int32_t z = prior_step_done();
   const int32_t i = 2 * (int32_t)(blockIdx.x * kPairThreads + threadIdx.x) + z;
@@ -701,6 +710,9 @@ __global__ void __launch_bounds__(kPairThreads, LBM_PAIR_MIN_BLOCKS)
         const uint32_t h = c_to_bits<PREC>(v[q], k.scale);
         out[q] = c ? out[q] | (h << 16) : h;
       }
+      if constexpr (KEEP_U)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) st_cs(u_out + j * ld + i + c, u[j]);
     }
   }
   unsigned short* dst16 = reinterpret_cast<unsigned short*>(dst);
@@ -713,10 +725,11 @@ __global__ void __launch_bounds__(kPairThreads, LBM_PAIR_MIN_BLOCKS)
 }
 
 // The same for the FP32 forms.
-template <int PREC, bool DAMPED>
+template <int PREC, bool DAMPED, bool KEEP_U>
 __global__ void __launch_bounds__(kPair32Threads, LBM_PAIR32_MIN_BLOCKS)
     sweep_pair32_kernel(const float* __restrict__ src, float* __restrict__ dst, Links links,
-                        int32_t n, int32_t ld, Coef<float> k, const float* __restrict__ alpha) {
+                        int32_t n, int32_t ld, Coef<float> k, const float* __restrict__ alpha,
+                        float* __restrict__ u_out) {
   static_assert(PREC == LBM_F32 || PREC == LBM_F32S, "FP32 forms only");
   const int32_t z = prior_step_done();
   const int32_t i = 2 * (int32_t)(blockIdx.x * kPair32Threads + threadIdx.x) + z;
@@ -736,17 +749,21 @@ __global__ void __launch_bounds__(kPair32Threads, LBM_PAIR32_MIN_BLOCKS)
     if (two) g[1][q + 1] = ld_nc(src + b);
   }
   if (i >= n) return;
-  float rho, u[3];
-  collide<float, DAMPED>(g[0], k, DAMPED ? ld_nc(alpha + i) : 0.f, rho, u);
+  float rho, u[2][3];
+  collide<float, DAMPED>(g[0], k, DAMPED ? ld_nc(alpha + i) : 0.f, rho, u[0]);
   if (two) {
-    collide<float, DAMPED>(g[1], k, DAMPED ? ld_nc(alpha + i + 1) : 0.f, rho, u);
+    collide<float, DAMPED>(g[1], k, DAMPED ? ld_nc(alpha + i + 1) : 0.f, rho, u[1]);
 #pragma unroll
-    for (int q = 0; q < 19; ++q)
-      asm volatile("st.global.cs.v2.f32 [%0], {%1, %2};" ::"l"(dst + q * ld + i), "f"(g[0][q]),
-                   "f"(g[1][q]) : "memory");
+    for (int q = 0; q < 19; ++q) st_cs_pair(dst + q * ld + i, g[0][q], g[1][q]);
+    if constexpr (KEEP_U)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) st_cs_pair(u_out + j * ld + i, u[0][j], u[1][j]);
   } else {
 #pragma unroll
     for (int q = 0; q < 19; ++q) st_cs(dst + q * ld + i, g[0][q]);
+    if constexpr (KEEP_U)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) st_cs(u_out + j * ld + i, u[0][j]);
   }
 }
 

@@ -140,32 +140,59 @@ namespace {
 // One step of a state from src to dst.  The lists that have short links take
 // two adjacent cells per thread in their plain FP32 and 16-bit steps; a list
 // of one wave loads its links before the wait.
+// u_out: keep the velocity there (a step that does not reduce).
 template <int PREC, bool DAMPED, bool SHORT>
 cudaError_t launch_step(const lbm_state* st, const typename Form<PREC>::S* src,
                         typename Form<PREC>::S* dst, const Links& links,
                         const Coef<typename Form<PREC>::C>& k, cudaStream_t stream, bool chained,
-                        bool reduce) {
+                        bool reduce, typename Form<PREC>::C* u_out) {
   const int32_t n = (int32_t)st->sp->n, ld = (int32_t)st->sp->ld;
-  const unsigned grid = (unsigned)st->nblocks;
   const auto* alpha = (const typename Form<PREC>::C*)st->alpha;
-  if (reduce)
-    return launch_sweep(sweep_kernel<PREC, DAMPED, kWarpSums, SHORT>, grid, stream, chained, src,
-                        dst, links, n, ld, k, alpha, st->partials);
+  const auto sweep = [&](auto* kernel) {
+    return launch_sweep(kernel, (unsigned)st->nblocks, stream, chained, src, dst, links, n, ld, k,
+                        alpha, st->partials, u_out);
+  };
+  const auto pair = [&](auto* kernel, int64_t threads) {
+    return launch_chained(kernel, (unsigned)((n + 2 * threads - 1) / (2 * threads)),
+                          (unsigned)threads, stream, chained, src, dst, links, n, ld, k, alpha,
+                          u_out);
+  };
+  if (reduce) return sweep(sweep_kernel<PREC, DAMPED, kWarpSums, SHORT>);
   if constexpr (SHORT && (PREC == LBM_F16S || PREC == LBM_BF16S)) {
-    constexpr int64_t cells = 2 * (int64_t)kPairThreads;
-    return launch_chained(sweep_pair_kernel<PREC, DAMPED>, (unsigned)((n + cells - 1) / cells),
-                          (unsigned)kPairThreads, stream, chained, src, dst, links, n, ld, k, alpha);
+    return u_out ? pair(sweep_pair_kernel<PREC, DAMPED, true>, kPairThreads)
+                 : pair(sweep_pair_kernel<PREC, DAMPED, false>, kPairThreads);
   } else if constexpr (SHORT && (PREC == LBM_F32 || PREC == LBM_F32S)) {
-    constexpr int64_t cells = 2 * (int64_t)kPair32Threads;
-    return launch_chained(sweep_pair32_kernel<PREC, DAMPED>, (unsigned)((n + cells - 1) / cells),
-                          (unsigned)kPair32Threads, stream, chained, src, dst, links, n, ld, k, alpha);
+    return u_out ? pair(sweep_pair32_kernel<PREC, DAMPED, true>, kPair32Threads)
+                 : pair(sweep_pair32_kernel<PREC, DAMPED, false>, kPair32Threads);
   } else {
     if constexpr (!SHORT && PREC != LBM_F64)
       if (st->one_wave)
-        return launch_sweep(sweep_kernel<PREC, DAMPED, kNoReduce, false, true>, grid, stream,
-                            chained, src, dst, links, n, ld, k, alpha, st->partials);
-    return launch_sweep(sweep_kernel<PREC, DAMPED, kNoReduce, SHORT>, grid, stream, chained, src,
-                        dst, links, n, ld, k, alpha, st->partials);
+        return u_out ? sweep(sweep_kernel<PREC, DAMPED, kKeepU, false, true>)
+                     : sweep(sweep_kernel<PREC, DAMPED, kNoReduce, false, true>);
+    return u_out ? sweep(sweep_kernel<PREC, DAMPED, kKeepU, SHORT>)
+                 : sweep(sweep_kernel<PREC, DAMPED, kNoReduce, SHORT>);
+  }
+}
+
+template <int PREC>
+auto step_of(const lbm_state* st) {
+  const bool wide = state_links(st->sp).wide != nullptr;
+  return wide ? (st->alpha ? launch_step<PREC, true, false> : launch_step<PREC, false, false>)
+              : (st->alpha ? launch_step<PREC, true, true> : launch_step<PREC, false, true>);
+}
+
+template <int PREC>
+cudaError_t plain_step(const lbm_state* st, const void* src, void* dst, void* u_out, double wp,
+                       double wm, const double F[3], cudaStream_t stream, bool chained) {
+  using S = typename Form<PREC>::S;
+  using C = typename Form<PREC>::C;
+  if constexpr (PREC == LBM_F64X) {
+    return launch_fx_step(st, (const double*)src, (double*)dst, u_out, wp, wm, F, stream, chained);
+  } else {
+    // steps in FP64 arithmetic are not chained (launch_steps)
+    return step_of<PREC>(st)(st, (const S*)src, (S*)dst, state_links(st->sp),
+                             make_coef<C>(wp, wm, F, st->scale_exp), stream,
+                             chained && PREC != LBM_F64, false, (C*)u_out);
   }
 }
 
@@ -178,8 +205,7 @@ int launch_steps(lbm_state* st, int32_t n_steps, double wp, double wm, const dou
     using S = typename Form<PREC>::S;
     const auto k = make_coef<typename Form<PREC>::C>(wp, wm, F, st->scale_exp);
     const Links links = state_links(st->sp);
-    const auto step = links.wide ? (st->alpha ? launch_step<PREC, true, false> : launch_step<PREC, false, false>)
-                                 : (st->alpha ? launch_step<PREC, true, true> : launch_step<PREC, false, true>);
+    const auto step = step_of<PREC>(st);
     for (int32_t t = 0; t < n_steps; ++t) {
       // Steps in FP64 arithmetic are not chained: a chained grid's blocks are
       // placed while the previous grid still holds its SMs, which packs
@@ -187,7 +213,7 @@ int launch_steps(lbm_state* st, int32_t n_steps, double wp, double wm, const dou
       // rate (32x32x64 bed: 2,333 against 2,580 MFLUP/s unchained).
       if (st->sp->n > 0)
         LBM_CUDA_TRY(step(st, (const S*)st->buf[st->cur], (S*)st->buf[st->cur ^ 1], links, k,
-                          stream, PREC != LBM_F64 && t > 0, reduce_last && t == n_steps - 1));
+                          stream, PREC != LBM_F64 && t > 0, reduce_last && t == n_steps - 1, nullptr));
       st->cur ^= 1;
     }
     return LBM_OK;
@@ -360,6 +386,12 @@ int dispatch_moments(const lbm_state* st, double* rho, double* u) {
 }
 
 }  // namespace
+
+cudaError_t launch_plain_step(const lbm_state* st, const void* src, void* dst, void* u_out,
+                              double wp, double wm, const double F[3], cudaStream_t stream,
+                              bool chained) {
+  LBM_DISPATCH(st->precision, plain_step, st, src, dst, u_out, wp, wm, F, stream, chained)
+}
 
 void free_state(lbm_state* st) {
   if (!st) return;
@@ -715,10 +747,10 @@ extern "C" int lbm_step_f64_noalloc(const double* f_src_dev, double* f_dst_dev,
   const Coef<double> k = make_coef<double>(omega_plus, omega_minus, force, 0);
   if (alpha_dev)
     sweep_kernel<LBM_F64, true, kBlockSums><<<(unsigned)nblocks, kSweepThreads, 0, stream>>>(
-        f_src_dev, f_dst_dev, Links{adj_dev, nullptr, nullptr}, n, n, k, alpha_dev, partials);
+        f_src_dev, f_dst_dev, Links{adj_dev, nullptr, nullptr}, n, n, k, alpha_dev, partials, nullptr);
   else
     sweep_kernel<LBM_F64, false, kBlockSums><<<(unsigned)nblocks, kSweepThreads, 0, stream>>>(
-        f_src_dev, f_dst_dev, Links{adj_dev, nullptr, nullptr}, n, n, k, nullptr, partials);
+        f_src_dev, f_dst_dev, Links{adj_dev, nullptr, nullptr}, n, n, k, nullptr, partials, nullptr);
   final_sum_kernel<<<1, 1024, 0, stream>>>(partials, nblocks, sums_dev);
   LBM_CUDA_TRY(cudaGetLastError());
   return LBM_OK;

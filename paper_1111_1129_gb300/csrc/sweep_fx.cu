@@ -34,6 +34,7 @@
 // through FP64; both are exact to FP64 round-off.  The
 // update is the TRT update of the FP64 form (same pair formulation), with
 // errors below FP64 round-off of f.
+#include "double_single.cuh"
 #include "lbm_kernels.cuh"
 
 namespace lbm {
@@ -294,13 +295,18 @@ __device__ __forceinline__ bool fx_damp(const int64_t* __restrict__ alpha_fx, in
   return true;
 }
 
+__device__ __forceinline__ void st_cs(float2* p, ds v) {
+  asm volatile("st.global.cs.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(v.hi), "f"(v.lo) : "memory");
+}
+
 // A step that does not reduce: n cells, PDF and link rows of stride ld.
-template <int HP_POW2, bool DAMPED, bool SHORT>
+// KEEP_U: the collision's velocity goes to u_out (3 rows of ld) as pairs.
+template <int HP_POW2, bool DAMPED, bool SHORT, bool KEEP_U>
 __global__ void __launch_bounds__(kFxThreads, LBM_FX_MIN_BLOCKS)
     sweep_fx_kernel(const double* __restrict__ src, double* __restrict__ dst, Links links,
                     int32_t n, int32_t ld, FxCoef k,
                     Coef<double> kd, const double* __restrict__ alpha,
-                    const int64_t* __restrict__ alpha_fx) {
+                    const int64_t* __restrict__ alpha_fx, float2* __restrict__ u_out) {
   const int32_t i = blockIdx.x * kFxThreads + threadIdx.x;
   prior_step_done();  // a chained launch waits here for the previous step
   int32_t idx[18];
@@ -311,12 +317,20 @@ __global__ void __launch_bounds__(kFxThreads, LBM_FX_MIN_BLOCKS)
     int64_t S[9], D[9], drho = 0, ux = 0, uy = 0, uz = 0, a1 = 0;
     if (fx_moments(b, k, S, D, drho, ux, uy, uz) &&
         fx_damp<DAMPED>(alpha_fx, n, i, k, ux, uy, uz, a1)) {
+      if constexpr (KEEP_U) {
+        st_cs(u_out + i, ds_from_fixed(ux, 58));
+        st_cs(u_out + ld + i, ds_from_fixed(uy, 58));
+        st_cs(u_out + 2 * ld + i, ds_from_fixed(uz, 58));
+      }
       fx_collide_store<HP_POW2>(S, D, drho, ux, uy, uz, k, a1, dst, ld, i);
     } else {
       double g[19], red[4];
 #pragma unroll
       for (int q = 0; q < 19; ++q) g[q] = __longlong_as_double(b[q]);
       fx_ieee_collide_store<DAMPED>(g, kd, DAMPED ? ld_nc(alpha + i) : 0.0, dst, ld, i, red);
+      if constexpr (KEEP_U)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) st_cs(u_out + j * ld + i, ds_from_double(red[1 + j]));
     }
   }
 }
@@ -398,28 +412,30 @@ FxCoef make_fx_coef(double wp, double wm, const double F[3], bool* pow2) {
 // reducing variant.
 template <int P2, bool DA, bool SHORT>
 cudaError_t launch_fx_form(const lbm_state* st, const double* src, double* dst,
-                           const Links& links, int32_t ld, const FxCoef& k,
-                           const Coef<double>& kd, cudaStream_t stream, bool chained,
-                           double* partials) {
-  const int32_t n = (int32_t)st->sp->n;
+                           const Links& links, const FxCoef& k, const Coef<double>& kd,
+                           cudaStream_t stream, bool chained, double* partials, float2* u_out) {
+  const int32_t n = (int32_t)st->sp->n, ld = (int32_t)st->sp->ld;
   const double* alpha = (const double*)st->alpha;
   const int64_t* afx = st->alpha_fx;
   if (partials)
     return launch_sweep(sweep_fx_reduce_kernel<P2, DA, SHORT>, (unsigned)st->nblocks, stream,
                         chained, src, dst, links, n, ld, k, kd, alpha, afx, partials);
-  return launch_chained(sweep_fx_kernel<P2, DA, SHORT>, (unsigned)((n + kFxThreads - 1) / kFxThreads),
-                        (unsigned)kFxThreads, stream, chained, src, dst, links, n, ld, k, kd, alpha,
-                        afx);
+  return launch_chained(u_out ? sweep_fx_kernel<P2, DA, SHORT, true> : sweep_fx_kernel<P2, DA, SHORT, false>,
+                        (unsigned)((n + kFxThreads - 1) / kFxThreads), (unsigned)kFxThreads,
+                        stream, chained, src, dst, links, n, ld, k, kd, alpha, afx, u_out);
 }
+// One fixed-point step of state st (its damping included) from src to dst;
+// partials non-null: the reducing variant; u_out non-null: the velocity is
+// kept.
 cudaError_t launch_fx(const lbm_state* st, const double* src, double* dst, const Links& links,
-                      int32_t ld, const FxCoef& k, bool pow2, const Coef<double>& kd,
-                      cudaStream_t stream, bool chained, double* partials) {
+                      const FxCoef& k, bool pow2, const Coef<double>& kd, cudaStream_t stream,
+                      bool chained, double* partials, float2* u_out) {
   const int p2 = !pow2 ? 0 : k.hp_sign;
 #define LBM_FX_FORM(P2, DA)                                                                  \
-  return links.wide ? launch_fx_form<P2, DA, false>(st, src, dst, links, ld, k, kd, stream,  \
-                                                    chained, partials)                       \
-                    : launch_fx_form<P2, DA, true>(st, src, dst, links, ld, k, kd, stream,   \
-                                                   chained, partials)
+  return links.wide ? launch_fx_form<P2, DA, false>(st, src, dst, links, k, kd, stream,      \
+                                                    chained, partials, u_out)                \
+                    : launch_fx_form<P2, DA, true>(st, src, dst, links, k, kd, stream,       \
+                                                   chained, partials, u_out)
   if (st->alpha) {
     if (p2 > 0) LBM_FX_FORM(1, true);
     if (p2 < 0) LBM_FX_FORM(-1, true);
@@ -444,24 +460,22 @@ int launch_steps_fx(lbm_state* st, int32_t n_steps, double wp, double wm, const 
     double* dst = (double*)st->buf[st->cur ^ 1];
     if (st->sp->n > 0) {
       const bool last = reduce_last && t == n_steps - 1;
-      LBM_CUDA_TRY(launch_fx(st, src, dst, links, (int32_t)st->sp->ld, k, pow2, kd,
-                             stream, t > 0, last ? st->partials : nullptr));
+      LBM_CUDA_TRY(launch_fx(st, src, dst, links, k, pow2, kd, stream, t > 0,
+                             last ? st->partials : nullptr, nullptr));
     }
     st->cur ^= 1;
   }
   return LBM_OK;
 }
 
-int launch_fx_step(const lbm_state* st, const double* src, double* dst, const int32_t* adj,
-                   int32_t ld, double wp, double wm, const double F[3], cudaStream_t stream,
-                   bool chained) {
-  if (st->sp->n == 0) return LBM_OK;
+cudaError_t launch_fx_step(const lbm_state* st, const double* src, double* dst, void* u_out,
+                           double wp, double wm, const double F[3], cudaStream_t stream,
+                           bool chained) {
+  if (st->sp->n == 0) return cudaSuccess;
   bool pow2 = false;
   const FxCoef k = make_fx_coef(wp, wm, F, &pow2);
-  const Coef<double> kd = make_coef<double>(wp, wm, F, 0);
-  LBM_CUDA_TRY(launch_fx(st, src, dst, Links{adj, nullptr, nullptr}, ld, k, pow2, kd, stream, chained,
-                         nullptr));
-  return LBM_OK;
+  return launch_fx(st, src, dst, state_links(st->sp), k, pow2, make_coef<double>(wp, wm, F, 0),
+                   stream, chained, nullptr, (float2*)u_out);
 }
 
 namespace {
