@@ -64,6 +64,20 @@ __host__ __device__ __forceinline__ double weight(int q) {
   return q == 0 ? 1.0 / 3.0 : (q <= 6 ? 1.0 / 18.0 : 1.0 / 36.0);
 }
 
+// Division of n < 2^31 by a fixed divisor: multiplication by ceil(2^(31+s) / d),
+// s = ceil(log2 d), exact for such n (Granlund and Montgomery 1994).
+struct FixedDiv {
+  uint32_t mul, shift;   // shift: 31 + s
+  __host__ __device__ __forceinline__ uint32_t of(uint32_t n) const {
+    return (uint32_t)(((uint64_t)n * mul) >> shift);
+  }
+};
+inline FixedDiv fixed_div(uint32_t d) {   // 1 <= d < 2^31
+  uint32_t s = 0;
+  while ((1ull << s) < d) ++s;
+  return {(uint32_t)(((1ull << (31 + s)) + d - 1) / d), 31 + s};
+}
+
 // Numbering-scheme key of box cell (x, y, z) (Sec. 3 "Numbering scheme").
 struct KeySpace {
   int32_t kind;
@@ -71,6 +85,14 @@ struct KeySpace {
   int64_t bx, by, bz, nbx, nby, nbz;
   int32_t hbits;  // Hilbert: bits per axis of the enclosing cube
   uint64_t size;  // every key is < size
+  // Curves (Morton, Hilbert): an aligned run of 8^levels keys, levels <= 4, is
+  // a cube of 2^levels cells per axis, walked along the curve of `levels` bits
+  // per axis turned by a signed permutation of the axes (curve_frame);
+  // unit[a]: the key of the unit vector along axis a on that small curve.
+  int32_t levels;
+  uint32_t unit[3];
+  // Blocked order with a key space below 2^31: the divisors of blocked_cell.
+  FixedDiv by_bsz, by_bx, by_bxy, by_nbx, by_nbxy;
 };
 
 // Hilbert curve on a 2^bits cube (Skilling, "Programming the Hilbert
@@ -109,26 +131,27 @@ __host__ __device__ inline uint64_t hilbert_encode(int bits, uint64_t x, uint64_
 }
 
 // Inverse of hilbert_encode: Gray-decode the transposed index, then redo
-// the level transformations from the bottom up.
-__host__ __device__ inline void hilbert_decode(int bits, uint64_t key, uint64_t& x, uint64_t& y,
-                                               uint64_t& z) {
-  uint64_t X[3] = {0, 0, 0};
+// the level transformations from the bottom up.  U: uint64_t, or uint32_t for
+// keys of at most 10 bits per axis.
+template <class U>
+__host__ __device__ inline void hilbert_decode(int bits, U key, U& x, U& y, U& z) {
+  U X[3] = {0, 0, 0};
   for (int lvl = 0; lvl < bits; ++lvl) {
-    X[0] |= ((key >> (3 * lvl + 2)) & 1ull) << lvl;
-    X[1] |= ((key >> (3 * lvl + 1)) & 1ull) << lvl;
-    X[2] |= ((key >> (3 * lvl)) & 1ull) << lvl;
+    X[0] |= ((key >> (3 * lvl + 2)) & (U)1) << lvl;
+    X[1] |= ((key >> (3 * lvl + 1)) & (U)1) << lvl;
+    X[2] |= ((key >> (3 * lvl)) & (U)1) << lvl;
   }
-  const uint64_t t0 = X[2] >> 1;
+  const U t0 = X[2] >> 1;
   X[2] ^= X[1];
   X[1] ^= X[0];
   X[0] ^= t0;
-  for (uint64_t q = 2; q != (1ull << bits); q <<= 1) {
-    const uint64_t p = q - 1;
+  for (U q = 2; q != ((U)1 << bits); q <<= 1) {
+    const U p = q - 1;
     for (int i = 2; i >= 0; --i) {
       if (X[i] & q) {
         X[0] ^= p;
       } else {
-        const uint64_t t = (X[0] ^ X[i]) & p;
+        const U t = (X[0] ^ X[i]) & p;
         X[0] ^= t;
         X[i] ^= t;
       }
@@ -248,6 +271,61 @@ __host__ __device__ inline bool cell_of(const KeySpace& ks, uint64_t k, int64_t&
     }
   }
   return k < ks.size && x < ks.nx && y < ks.ny && z < ks.nz;
+}
+
+// cell_of in blocked order, for a key space below 2^31: five multiplications
+// instead of seven divisions.
+__host__ __device__ inline bool blocked_cell(const KeySpace& ks, uint32_t k, int32_t& x, int32_t& y,
+                                             int32_t& z) {
+  const uint32_t bx = (uint32_t)ks.bx, by = (uint32_t)ks.by, nbx = (uint32_t)ks.nbx,
+                 nby = (uint32_t)ks.nby;
+  const uint32_t blk = ks.by_bsz.of(k), loc = k - blk * (bx * by * (uint32_t)ks.bz);
+  const uint32_t lyz = ks.by_bx.of(loc), lz = ks.by_bxy.of(loc);
+  const uint32_t biyz = ks.by_nbx.of(blk), biz = ks.by_nbxy.of(blk);
+  x = (int32_t)((blk - biyz * nbx) * bx + (loc - lyz * bx));
+  y = (int32_t)((biyz - biz * nby) * by + (lyz - lz * by));
+  z = (int32_t)(biz * (uint32_t)ks.bz + lz);
+  return k < ks.size && x < ks.nx && y < ks.ny && z < ks.nz;
+}
+
+inline bool is_curve(int32_t kind) {
+  return kind == LBM_ORDER_MORTON1 || kind == LBM_ORDER_MORTON2 || kind == LBM_ORDER_HILBERT;
+}
+
+// Where and how a curve walks its aligned cube number `tile` of 8^levels keys:
+// the key 8^levels tile + l is the cell at + c[0] d[0] + c[1] d[1] + c[2] d[2],
+// c = curve_local(l).
+struct CurveFrame {
+  int32_t at[3], d[3][3];
+};
+// Column `which` of the frame: 0 its start, 1..3 the images of the unit vectors
+// (still to be taken relative to the start).
+__host__ __device__ inline void curve_point(const KeySpace& ks, uint64_t tile, int which,
+                                            int32_t p[3]) {
+  int64_t x, y, z;
+  cell_of(ks, (tile << (3 * ks.levels)) + (which ? ks.unit[which - 1] : 0u), x, y, z);
+  p[0] = (int32_t)x;
+  p[1] = (int32_t)y;
+  p[2] = (int32_t)z;
+}
+// The cell of local key l < 8^levels on the small curve.
+__host__ __device__ inline void curve_local(const KeySpace& ks, uint32_t l, uint32_t c[3]) {
+  if (ks.kind == LBM_ORDER_HILBERT) {
+    hilbert_decode<uint32_t>(ks.levels, l, c[0], c[1], c[2]);
+    return;
+  }
+  for (int a = 0; a < 3; ++a) {
+    c[a] = 0;
+    if (ks.kind == LBM_ORDER_MORTON1) {
+      for (int b = 0; b < 4; ++b) c[a] |= ((l >> (3 * b + a)) & 1u) << b;
+    } else {
+      for (int g = 0; g < 2; ++g) c[a] |= ((l >> (6 * g + 2 * a)) & 3u) << (2 * g);
+    }
+  }
+}
+__host__ __device__ inline void curve_cell(const CurveFrame& f, const uint32_t c[3], int32_t p[3]) {
+  for (int a = 0; a < 3; ++a)
+    p[a] = f.at[a] + (int32_t)c[0] * f.d[0][a] + (int32_t)c[1] * f.d[1][a] + (int32_t)c[2] * f.d[2][a];
 }
 
 // Validates dims/ordering and fills the key space; returns LBM_OK or an error.
