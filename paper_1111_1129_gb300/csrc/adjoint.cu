@@ -67,8 +67,7 @@ struct lbm_adjoint {
   bool fresh;       // lam[0], part, dalpha, u and last are as the forward pass left them
   double* part;     // [nblocks][4]: dJ/dF_x, dJ/dF_y, dJ/dF_z, sum u_axis
   double* dalpha;   // [N]
-  double* red_dev;  // [4]
-  double* red_host; // [4], pinned
+  double* red_host; // [4], pinned, written by final_sum_kernel
   cudaEvent_t done;
   int have_forward;
   double wp, wm, F[3];
@@ -750,10 +749,8 @@ int finish_sums(lbm_adjoint* ad) {
     for (int j = 0; j < 4; ++j) ad->red_host[j] = 0.0;
     return LBM_OK;
   }
-  final_sum_kernel<<<1, 1024, 0, stream>>>(ad->part, ad->st->nblocks, ad->red_dev);
+  final_sum_kernel<<<1, 1024, 0, stream>>>(ad->part, ad->st->nblocks, ad->red_host);
   LBM_CUDA_TRY(cudaGetLastError());
-  LBM_CUDA_TRY(cudaMemcpyAsync(ad->red_host, ad->red_dev, 4 * sizeof(double),
-                               cudaMemcpyDeviceToHost, stream));
   return wait_event(ad->done, stream, 0.0);
 }
 
@@ -766,7 +763,7 @@ void free_adjoint(lbm_adjoint* ad) {
   const cudaStream_t s = ad->stream;
   cudaStreamSynchronize(s);
   for (void* p : {ad->ckpt, ad->f[0], ad->f[1], ad->u, ad->lam[0], ad->lam[1], (void*)ad->part,
-                  (void*)ad->dalpha, (void*)ad->red_dev})
+                  (void*)ad->dalpha})
     dev_free(p, s, false);
   if (ad->red_host) cudaFreeHost(ad->red_host);
   if (ad->done) cudaEventDestroy(ad->done);
@@ -821,7 +818,6 @@ extern "C" int lbm_adjoint_create(const lbm_state* st, int32_t n_steps, int32_t 
             rows(&ad->lam[0], 19, crow) && rows(&ad->lam[1], 19, crow) &&
             dev_alloc(&ad->part, sizeof(double) * 4 * st->nblocks, s, false) == cudaSuccess &&
             dev_alloc(&ad->dalpha, sizeof(double) * n, s, false) == cudaSuccess &&
-            dev_alloc(&ad->red_dev, sizeof(double) * 4, s, false) == cudaSuccess &&
             cudaMallocHost(&ad->red_host, sizeof(double) * 4) == cudaSuccess &&
             cudaEventCreateWithFlags(&ad->done, cudaEventDisableTiming) == cudaSuccess;
   if (!ok) {

@@ -866,10 +866,8 @@ int batch_reduce(lbm_state* st, int32_t axis, double* mass_out, double* flux_out
   const cudaStream_t stream = st->sp->stream;
   if (st->sp->n > 0) {
     batch_final_kernel<<<b->n_beds, 1024, 0, stream>>>(st->partials, b->d_begin, b->d_count,
-                                                       b->d_red);
+                                                       b->h_red);
     LBM_CUDA_TRY(cudaGetLastError());
-    LBM_CUDA_TRY(cudaMemcpyAsync(b->h_red, b->d_red, sizeof(double) * 4 * b->n_beds,
-                                 cudaMemcpyDeviceToHost, stream));
     int rc = wait_event(st->done, stream, 0.0);
     if (rc == LBM_OK) rc = take_barrier_error(st, stream);
     if (rc != LBM_OK) return rc;
@@ -897,7 +895,7 @@ void free_batch(lbm_state* st) {
   const cudaStream_t stream = st->stream;
   cudaStreamSynchronize(stream);
   for (void* p : {(void*)b->d_begin, (void*)b->d_count, (void*)b->d_chunk_bed, b->d_force,
-                  (void*)b->d_red, (void*)b->d_sync, (void*)b->d_sync_err})
+                  (void*)b->d_sync, (void*)b->d_sync_err})
     dev_free(p, stream, false);
   free_group_tables(b, stream);
   for (void* p : {b->h_force, (void*)b->h_red, (void*)b->h_sync_err})
@@ -999,7 +997,6 @@ extern "C" int lbm_state_create_batched(const lbm_sparse* const* beds, int32_t n
                 cudaSuccess &&
             dev_alloc(&b->d_force, fbytes * n_beds, stream, false) == cudaSuccess &&
             cudaMallocHost(&b->h_force, fbytes * n_beds) == cudaSuccess &&
-            dev_alloc(&b->d_red, sizeof(double) * 4 * n_beds, stream, false) == cudaSuccess &&
             cudaMallocHost(&b->h_red, sizeof(double) * 4 * n_beds) == cudaSuccess &&
             dev_alloc(&b->d_sync, sizeof(uint32_t) * (size_t)(n_chunks + 1), stream, false) ==
                 cudaSuccess &&

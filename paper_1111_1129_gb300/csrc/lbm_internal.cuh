@@ -411,8 +411,7 @@ struct Batch {
   int32_t* d_chunk_bed;  // [n_pad / kBatchChunk] bed of each chunk
   void* d_force;         // [n_beds] per-bed force constants (arithmetic type)
   void* h_force;         // pinned staging for d_force
-  double* d_red;         // [n_beds][4] per-bed final sums
-  double* h_red;         // pinned
+  double* h_red;         // [n_beds][4] per-bed final sums, pinned, written by the device
   int block, cpt;        // launch configuration of the non-reducing steps
   cudaStream_t capture;  // private stream used to capture graphs
   cudaGraphExec_t graph; // cached K-step graph (or null)
@@ -502,8 +501,8 @@ struct lbm_state {
                        // then [nblocks * 4] room for the group values of lbm_reduce_flux
   int64_t nblocks;
   bool one_wave;       // at most one_wave_cells(): plain FP32/16-bit steps load links first
-  double* red_dev;     // [4] final sums
-  double* red_host;    // [4] pinned
+  unsigned* arrived;   // CTAs of the running flux_sums_kernel that are done
+  double* red_host;    // [4] pinned, written by flux_sums_kernel
   int64_t steps;
   double last_force[3];
   double last_wp, last_wm;

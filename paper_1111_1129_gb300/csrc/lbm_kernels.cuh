@@ -413,7 +413,7 @@ __device__ __forceinline__ void store_warp_sums(const double w[4], double* parti
 }
 
 // Combines the block's warp sums in warp order into out[0..3] (the value
-// collapse_warp_sums_kernel forms from store_warp_sums slots); has a block
+// flux_sums_kernel forms from store_warp_sums slots); has a block
 // barrier.
 __device__ __forceinline__ void store_block_sums(const double w[4], double* out) {
   __shared__ double sm[kWarpsPerBlock][4];
@@ -790,17 +790,34 @@ __global__ void __launch_bounds__(kSweepThreads)
   u_out[2 * (int64_t)n + i] = (double)u[2];
 }
 
-// Group values from per-warp slots: thread b forms block b's value (its
-// kWarpsPerBlock slots in slot order, the value store_block_sums forms
-// inside a block), and each 256-thread CTA adds its
-// 256 block values by a fixed tree into groups[4 g + j].  final_sum_kernel
-// then adds the ceil(nblocks / 256) groups.  One 1024-thread block reading
-// all block values had cost 0.15 ms per call on the 1024x256x256 bed.
+// Sum of 1024 values v[0..1023] by a fixed tree, four of each, in a block of
+// THREADS: sm is left with the sums in sm[0].
+template <int THREADS>
+__device__ __forceinline__ void tree_sum_1024(double (*sm)[4]) {
+  __syncthreads();
+  for (int s = 512; s > 0; s >>= 1) {
+    for (int t = threadIdx.x; t < s; t += THREADS)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) sm[t][j] += sm[t + s][j];
+    __syncthreads();
+  }
+}
+
+// The flux sums of a step from its per-warp slots, in one launch.  Thread b
+// forms block b's value (its kWarpsPerBlock slots in slot order, the value
+// store_block_sums forms inside a block); each 256-thread CTA adds its 256
+// block values by a fixed tree into groups[4 g + j]; and the last CTA to arrive
+// adds the group values in the order of final_sum_kernel and writes the four
+// sums to `out`, which may be pinned host memory, so that nothing is copied.
+// One 1024-thread block reading all block values had cost 0.15 ms per call on
+// the 1024x256x256 bed; two kernels and a copy cost a short call two launches.
+// *arrived counts the CTAs and wraps to 0.
 constexpr int kCollapseThreads = 256;
 __global__ void __launch_bounds__(kCollapseThreads)
-    collapse_warp_sums_kernel(const double* __restrict__ part, int64_t nblocks,
-                              double* __restrict__ groups) {
-  __shared__ double sm[kCollapseThreads][4];
+    flux_sums_kernel(const double* __restrict__ part, int64_t nblocks, double* groups,
+                     unsigned* arrived, double* out) {
+  __shared__ double sm[1024][4];
+  __shared__ bool last;
   const int64_t b = (int64_t)blockIdx.x * kCollapseThreads + threadIdx.x;
   double v[4] = {0.0, 0.0, 0.0, 0.0};
   if (b < nblocks) {
@@ -820,6 +837,22 @@ __global__ void __launch_bounds__(kCollapseThreads)
     __syncthreads();
   }
   if (threadIdx.x < 4) groups[4 * blockIdx.x + threadIdx.x] = sm[0][threadIdx.x];
+  __threadfence();   // the group's value before the arrival
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicInc(arrived, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();   // the arrivals before the groups' values
+  for (int t = threadIdx.x; t < 1024; t += kCollapseThreads) {
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    for (unsigned g = (unsigned)t; g < gridDim.x; g += 1024)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[j] += __ldcg(groups + 4 * (int64_t)g + j);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) sm[t][j] = acc[j];
+  }
+  tree_sum_1024<kCollapseThreads>(sm);
+  if (threadIdx.x < 4) out[threadIdx.x] = sm[0][threadIdx.x];
 }
 
 // Final fixed-order sum of the block values: out[j] = sum_b part[4 b + j].
@@ -832,13 +865,7 @@ __global__ void __launch_bounds__(1024)
     for (int j = 0; j < 4; ++j) acc[j] += part[4 * b + j];
 #pragma unroll
   for (int j = 0; j < 4; ++j) sm[threadIdx.x][j] = acc[j];
-  __syncthreads();
-  for (int s = 512; s > 0; s >>= 1) {
-    if (threadIdx.x < s)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) sm[threadIdx.x][j] += sm[threadIdx.x + s][j];
-    __syncthreads();
-  }
+  tree_sum_1024<1024>(sm);
   if (threadIdx.x < 4) out[threadIdx.x] = sm[0][threadIdx.x];
 }
 

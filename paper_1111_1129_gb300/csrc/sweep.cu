@@ -120,6 +120,9 @@ static double g_timeout_s = 600.0;
 int wait_event(cudaEvent_t ev, cudaStream_t stream, double timeout_s) {
   LBM_CUDA_TRY(cudaEventRecord(ev, stream));
   const double limit = timeout_s > 0 ? timeout_s : g_timeout_s;
+  // A sleep lasts 70 us or more, as long as a short call; the first 200 us are
+  // polled without one.
+  constexpr double kPollS = 200e-6;
   const auto t0 = std::chrono::steady_clock::now();
   for (;;) {
     const cudaError_t e = cudaEventQuery(ev);
@@ -129,7 +132,7 @@ int wait_event(cudaEvent_t ev, cudaStream_t stream, double timeout_s) {
         std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     if (el > limit)
       return fail(LBM_ETIMEOUT, "queued work still running after %.1f s", limit);
-    std::this_thread::sleep_for(std::chrono::microseconds(20));
+    if (el > kPollS) std::this_thread::sleep_for(std::chrono::microseconds(20));
   }
 }
 
@@ -400,7 +403,7 @@ void free_state(lbm_state* st) {
   const cudaStream_t s = st->stream;
   cudaStreamSynchronize(s);
   for (void* p : {st->buf[0], st->buf[1], st->alpha, (void*)st->alpha_fx, (void*)st->partials,
-                  (void*)st->red_dev})
+                  (void*)st->arrived})
     dev_free(p, s, false);
   if (st->red_host) cudaFreeHost(st->red_host);
   if (st->done) cudaEventDestroy(st->done);
@@ -445,7 +448,7 @@ extern "C" int lbm_state_create(const lbm_sparse* sp, int32_t precision, int32_t
             dev_alloc(&st->buf[1], bytes, stream, false) == cudaSuccess &&
             dev_alloc(&st->partials, sizeof(double) * 4 * (kWarpsPerBlock + 1) * st->nblocks,
                       stream, false) == cudaSuccess &&
-            dev_alloc(&st->red_dev, sizeof(double) * 4, stream, false) == cudaSuccess &&
+            dev_alloc(&st->arrived, sizeof(unsigned), stream, false) == cudaSuccess &&
             cudaMallocHost(&st->red_host, sizeof(double) * 4) == cudaSuccess &&
             cudaEventCreateWithFlags(&st->done, cudaEventDisableTiming) == cudaSuccess;
   if (!ok) {
@@ -454,6 +457,10 @@ extern "C" int lbm_state_create(const lbm_sparse* sp, int32_t precision, int32_t
     return fail(LBM_ENOMEM, "state allocation of 2 x %zu bytes failed", bytes);
   }
   int rc = dispatch_set(st, nullptr, 1);
+  if (rc == LBM_OK) {
+    const cudaError_t e = cudaMemsetAsync(st->arrived, 0, sizeof(unsigned), stream);
+    if (e != cudaSuccess) rc = cuda_fail(e, "cudaMemsetAsync");
+  }
   // The first step writes every slot of the second grid before anything
   // reads it.  A concatenated batch (ord.kind -1) also has padding cells
   // that no step writes: zero its second grid so that they read back as 0.
@@ -625,12 +632,9 @@ extern "C" int lbm_reduce_flux(lbm_state* st, int32_t axis, double* mass_out, do
     // group sums after the warp slots (room for nblocks values of 4)
     double* groups = st->partials + 4 * kWarpsPerBlock * st->nblocks;
     const int64_t ngroups = (st->nblocks + kCollapseThreads - 1) / kCollapseThreads;
-    collapse_warp_sums_kernel<<<(unsigned)ngroups, kCollapseThreads, 0, stream>>>(
-        st->partials, st->nblocks, groups);
-    final_sum_kernel<<<1, 1024, 0, stream>>>(groups, ngroups, st->red_dev);
+    flux_sums_kernel<<<(unsigned)ngroups, kCollapseThreads, 0, stream>>>(
+        st->partials, st->nblocks, groups, st->arrived, st->red_host);
     LBM_CUDA_TRY(cudaGetLastError());
-    LBM_CUDA_TRY(cudaMemcpyAsync(st->red_host, st->red_dev, sizeof(double) * 4,
-                                 cudaMemcpyDeviceToHost, stream));
     const int rc = wait_event(st->done, stream, 0.0);
     if (rc != LBM_OK) return rc;
   } else {
