@@ -460,8 +460,10 @@ void lbm_free(void* handle);
 
 /* ---- device memory --------------------------------------------------------
  * Handles take their device memory from a caller-supplied allocator when
- * one is set, else from cudaMalloc (cudaMallocAsync on the handle's stream
- * for the sparse representation and its scratch).
+ * one is set, else from cudaMalloc, for the sparse representation and its
+ * scratch from a stream-ordered pool of the library that keeps up to 1/64 of
+ * the device's memory for the next lattice; a call of this function gives
+ * back what it keeps.
  *   alloc(bytes, stream, ctx) returns a device pointer aligned to at least
  *     16 bytes (cudaMalloc and PyTorch's allocator give 256), or NULL: the
  *     calling function then fails with LBM_ENOMEM.  A pointer aligned to

@@ -3,6 +3,7 @@
 #include <atomic>
 #include <cstdarg>
 #include <cstdio>
+#include <mutex>
 #include <string>
 
 #include "lbm_internal.cuh"
@@ -17,6 +18,62 @@ lbm_alloc_fn g_alloc = nullptr;
 lbm_free_fn g_release = nullptr;
 void* g_alloc_ctx = nullptr;
 std::atomic<int64_t> g_live{0};
+
+// Ordered blocks of the library's own come from one pool per device, which
+// keeps up to 1/64 of the device's memory (4.4 GB on GB300) mapped when it is
+// free: mapping fresh pages and giving them back took three quarters of the
+// time of assembling a large lattice (1024x256x256 bed with its outputs 11.9
+// ms, 2.8 ms with the pool).  Memory beyond that goes back to the device when the
+// stream is next synchronised; all of it when an allocation of the library
+// fails or lbm_set_allocator is called.  The driver orders the reuse of a block
+// across streams, and the calls are safe from several threads.
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mutex;
+cudaMemPool_t g_pool[kMaxDevices] = {};
+
+// The current device's pool, or null (then the device's default pool serves).
+cudaMemPool_t device_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  if (!g_pool[dev]) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess &&
+        cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
+      uint64_t keep = total / 64;
+      if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+        g_pool[dev] = pool;
+      else cudaMemPoolDestroy(pool);
+    }
+    if (!g_pool[dev]) cudaGetLastError();
+  }
+  return g_pool[dev];
+}
+
+void give_back_pools() {
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  for (cudaMemPool_t pool : g_pool)
+    if (pool) cudaMemPoolTrimTo(pool, 0);
+}
+
+cudaError_t own_alloc(void** p, size_t bytes, cudaStream_t stream, bool ordered) {
+  cudaMemPool_t pool = ordered ? device_pool() : nullptr;
+  const auto get = [&]() {
+    return pool      ? cudaMallocFromPoolAsync(p, bytes, pool, stream)
+           : ordered ? cudaMallocAsync(p, bytes, stream)
+                     : cudaMalloc(p, bytes);
+  };
+  const cudaError_t e = get();
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  give_back_pools();
+  return get();
+}
 }
 
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t stream, bool ordered) {
@@ -30,7 +87,7 @@ cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t stream, bool ordered)
     }
     *p = q;
   } else {
-    const cudaError_t e = ordered ? cudaMallocAsync(p, bytes, stream) : cudaMalloc(p, bytes);
+    const cudaError_t e = own_alloc(p, bytes, stream, ordered);
     if (e != cudaSuccess) {
       *p = nullptr;
       return e;
@@ -96,6 +153,7 @@ extern "C" int lbm_set_allocator(lbm_alloc_fn alloc, lbm_free_fn release, void* 
   if (live != 0)
     return lbm::fail(LBM_EINVAL, "%lld device blocks of existing handles are still live",
                      (long long)live);
+  lbm::give_back_pools();
   lbm::g_alloc = alloc;
   lbm::g_release = release;
   lbm::g_alloc_ctx = ctx;

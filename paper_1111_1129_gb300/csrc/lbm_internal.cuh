@@ -20,8 +20,8 @@ int fail(int status, const char* fmt, ...);
 int cuda_fail(cudaError_t e, const char* what);
 void clear_error();
 // Device memory of every handle: the caller's allocator when one is set
-// (lbm_set_allocator), else cudaMallocAsync / cudaFreeAsync on `stream`
-// (ordered) or cudaMalloc / cudaFree.  An unordered free expects the work
+// (lbm_set_allocator), else the library's pool (ordered on `stream`) or
+// cudaMalloc / cudaFree.  An unordered free expects the work
 // on the block to have finished.
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t stream, bool ordered);
 void dev_free(void* p, cudaStream_t stream, bool ordered);
