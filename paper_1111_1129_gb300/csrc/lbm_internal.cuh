@@ -532,6 +532,11 @@ cudaError_t launch_plain_step(const lbm_state* st, const void* src, void* dst, v
 cudaError_t launch_fx_step(const lbm_state* st, const double* src, double* dst, void* u_out,
                            double wp, double wm, const double F[3], cudaStream_t stream,
                            bool chained);
+
+// rho [n] and u [3][n] of the step that pulled from src (rows of stride ld)
+// under force F, for the FP64 forms.
+cudaError_t launch_moments_fx(const lbm_state* st, const double* src, const double F[3],
+                              double* rho, double* u);
 // Fills the fixed-point damping rows (alpha_fx) of an FP64-storage state
 // from FP64 alpha on the device.
 int set_alpha_fx(lbm_state* st, const double* alpha_dev);

@@ -51,11 +51,49 @@ struct RestRow {
   typename Form<PREC>::S v[19];
 };
 
+// FP32 to FP64 and back, rounding to nearest even, in integer instructions: a
+// conversion issues at the FP64 rate, 1/64 of the FP32 rate.  Two FP64
+// instructions a value, the conversion and the add of the weight, had bound
+// the copies of the FP32 and 16-bit forms (36.1 million cells of FP16 to FP64
+// 2,541 us, 1,376 us now; 11.6 million of FP32 832 us, 466 us now; 1.03 and
+// 0.40 ms at the copy rate).  Subnormal results, infinities and NaN take the
+// instruction.
+__device__ __noinline__ double widen_any(float v) { return (double)v; }
+__device__ __noinline__ float narrow_any(double v) { return (float)v; }
+
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t u = __float_as_uint(v), mag = u & 0x7fffffffu;
+  if (mag - 0x00800000u >= 0x7f000000u && mag != 0) return widen_any(v);
+  const uint32_t hi = mag ? (mag >> 3) + (896u << 20) : 0u;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
+template <class C>
+__device__ __forceinline__ C narrow(double v) {
+  if constexpr (sizeof(C) == 8) {
+    return v;
+  } else {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t mag = hi & 0x7fffffffu;
+    if (mag - (897u << 20) >= (254u << 20) && (mag | lo) != 0) return narrow_any(v);
+    // a carry out of the mantissa raises the exponent, up to infinity, as it must
+    const uint32_t t = ((mag - (896u << 20)) << 3) | (lo >> 29);
+    const uint32_t r = t + (((lo & 0x1fffffffu) + 0x0fffffffu + (t & 1u)) >> 29);
+    return __uint_as_float(((mag | lo) ? r : 0u) | (hi & 0x80000000u));
+  }
+}
+
+// A block of the row kernels takes UNROLL stretches of kRowThreads values of a
+// row at a time: kRowUnroll in flight per thread where the grid is full, one
+// where a list is too short for that (n <= kRowThreads kRowBlocks).
+constexpr int kRowThreads = 256, kRowBlocks = 2048, kRowUnroll = 4;
+
 // One row q = blockIdx.y per grid row, so no slot index is divided by N.
 // From rest the stored value comes from `rest`; from f the value is
 // converted as the form stores it (the deviation f - w in FP64, then
 // rounded).  f is [19][n]; dst has rows of stride ld.
-template <int PREC>
+template <int PREC, int UNROLL>
 __global__ void set_pdfs_kernel(typename Form<PREC>::S* __restrict__ dst,
                                 const double* __restrict__ f, int32_t n, int32_t ld, double scale,
                                 RestRow<PREC> rest) {
@@ -63,39 +101,56 @@ __global__ void set_pdfs_kernel(typename Form<PREC>::S* __restrict__ dst,
   using C = typename Form<PREC>::C;
   const double w = weight(q);
   const typename Form<PREC>::S r = rest.v[q];
+  typename Form<PREC>::S* to = dst + (int64_t)q * ld;
   // a grid-stride loop: one-element threads made this kernel bound by
   // block scheduling (2.9 ms for 1.25 GB)
-  for (int32_t i = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x); i < n;
-       i += (int32_t)(gridDim.x * blockDim.x)) {
-    const int64_t t = (int64_t)q * ld + i;
-    if (!f) {
-      dst[t] = r;
-    } else {
-      const double fv = f[(int64_t)q * n + i];
-      C c;
-      if constexpr (Form<PREC>::kShifted) c = (C)(fv - w);
-      else c = (C)fv;
-      dst[t] = encode<PREC>(c, (C)scale);
-    }
+  if (!f) {
+    for (int32_t i = (int32_t)(blockIdx.x * kRowThreads + threadIdx.x); i < n;
+         i += (int32_t)(gridDim.x * kRowThreads))
+      to[i] = r;
+    return;
+  }
+  const double* from = f + (int64_t)q * n;
+  for (int64_t i0 = (int64_t)blockIdx.x * (kRowThreads * UNROLL) + threadIdx.x; i0 < n;
+       i0 += (int64_t)gridDim.x * (kRowThreads * UNROLL)) {
+    double v[UNROLL];
+#pragma unroll
+    for (int j = 0; j < UNROLL; ++j)
+      v[j] = from[i0 + j * kRowThreads < n ? i0 + j * kRowThreads : i0];
+#pragma unroll
+    for (int j = 0; j < UNROLL; ++j)
+      if (i0 + j * kRowThreads < n)
+        to[i0 + j * kRowThreads] =
+            encode<PREC>(narrow<C>(Form<PREC>::kShifted ? v[j] - w : v[j]), (C)scale);
   }
 }
 
 // The inverse of set_pdfs_kernel from f: src rows of stride ld, f [19][n].
-template <int PREC>
+template <int PREC, int UNROLL>
 __global__ void get_pdfs_kernel(const typename Form<PREC>::S* __restrict__ src, double* f,
                                 int32_t n, int32_t ld, double inv_scale) {
   const int q = (int)blockIdx.y;
   using C = typename Form<PREC>::C;
   const double w = weight(q);
-  for (int32_t i = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x); i < n;
-       i += (int32_t)(gridDim.x * blockDim.x)) {
-    const double v = (double)decode<PREC>(src[(int64_t)q * ld + i], (C)inv_scale);
-    f[(int64_t)q * n + i] = Form<PREC>::kShifted ? w + v : v;
+  const typename Form<PREC>::S* from = src + (int64_t)q * ld;
+  double* to = f + (int64_t)q * n;
+  for (int64_t i0 = (int64_t)blockIdx.x * (kRowThreads * UNROLL) + threadIdx.x; i0 < n;
+       i0 += (int64_t)gridDim.x * (kRowThreads * UNROLL)) {
+    typename Form<PREC>::S v[UNROLL];
+#pragma unroll
+    for (int j = 0; j < UNROLL; ++j)
+      v[j] = from[i0 + j * kRowThreads < n ? i0 + j * kRowThreads : i0];
+#pragma unroll
+    for (int j = 0; j < UNROLL; ++j)
+      if (i0 + j * kRowThreads < n) {
+        const double d = widen(decode<PREC>(v[j], (C)inv_scale));
+        to[i0 + j * kRowThreads] = Form<PREC>::kShifted ? w + d : d;
+      }
   }
 }
 
-// Grid of the row kernels above: x blocks of 256 threads per row, 19 rows.
-dim3 row_grid(int64_t n) { return dim3((unsigned)std::min<int64_t>((n + 255) / 256, 2048), 19); }
+// Grid of the row kernels above: x blocks of kRowThreads threads per row, 19 rows.
+dim3 row_grid(int64_t n) { return dim3((unsigned)std::min<int64_t>((n + kRowThreads - 1) / kRowThreads, kRowBlocks), 19); }
 
 template <class C>
 __global__ void set_alpha_kernel(C* dst, const double* a, int32_t n) {
@@ -122,7 +177,7 @@ int wait_event(cudaEvent_t ev, cudaStream_t stream, double timeout_s) {
   const double limit = timeout_s > 0 ? timeout_s : g_timeout_s;
   // A sleep lasts 70 us or more, as long as a short call; so the first 4 ms
   // are polled without one, and later it is at most 2% of the wait.  (32x32x64
-  // bed, one step with its sums and fields: 145 us when every poll slept, 57
+  // bed, one step with its sums and fields: 145 us when every poll slept, 58
   // us now, with the sums in one launch.)
   constexpr double kPollS = 4e-3;
   const auto t0 = std::chrono::steady_clock::now();
@@ -135,7 +190,6 @@ int wait_event(cudaEvent_t ev, cudaStream_t stream, double timeout_s) {
     if (el > limit)
       return fail(LBM_ETIMEOUT, "queued work still running after %.1f s", limit);
     if (el > kPollS) std::this_thread::sleep_for(std::chrono::microseconds(20));
-    else std::this_thread::yield();
   }
 }
 
@@ -234,13 +288,17 @@ int launch_moments(const lbm_state* st, double* rho, double* u) {
   if (n == 0) return LBM_OK;
   const Coef<C> k = make_coef<C>(st->last_wp, st->last_wm, st->last_force, st->scale_exp);
   const S* prev = (const S*)st->buf[st->cur ^ 1];
-  const C* alpha = (const C*)st->alpha;
-  const Links links = state_links(st->sp);
-  const auto kernel = links.wide ? (alpha ? moments_kernel<PREC, true, false> : moments_kernel<PREC, false, false>)
-                                 : (alpha ? moments_kernel<PREC, true, true> : moments_kernel<PREC, false, true>);
-  kernel<<<(unsigned)st->nblocks, kSweepThreads, 0, st->sp->stream>>>(
-      prev, links, n, (int32_t)st->sp->ld, k, alpha, rho, u);
-  LBM_CUDA_TRY(cudaGetLastError());
+  if constexpr (sizeof(C) == 8) {
+    LBM_CUDA_TRY(launch_moments_fx(st, prev, st->last_force, rho, u));
+  } else {
+    const C* alpha = (const C*)st->alpha;
+    const Links links = state_links(st->sp);
+    const auto kernel = links.wide ? (alpha ? moments_kernel<PREC, true, false> : moments_kernel<PREC, false, false>)
+                                   : (alpha ? moments_kernel<PREC, true, true> : moments_kernel<PREC, false, true>);
+    kernel<<<(unsigned)st->nblocks, kSweepThreads, 0, st->sp->stream>>>(
+        prev, links, n, (int32_t)st->sp->ld, k, alpha, rho, u);
+    LBM_CUDA_TRY(cudaGetLastError());
+  }
   return LBM_OK;
 }
 
@@ -264,7 +322,8 @@ int launch_set(lbm_state* st, const double* f, int from_rest) {
     }
   }
   const int32_t n = (int32_t)st->sp->n;
-  set_pdfs_kernel<PREC><<<row_grid(n), 256, 0, st->sp->stream>>>(
+  const auto kernel = n <= kRowThreads * kRowBlocks ? set_pdfs_kernel<PREC, 1> : set_pdfs_kernel<PREC, kRowUnroll>;
+  kernel<<<row_grid(n), kRowThreads, 0, st->sp->stream>>>(
       (S*)st->buf[grouped ? st->cur ^ 1 : st->cur], from_rest ? nullptr : f, n,
       (int32_t)st->sp->ld, std::ldexp(1.0, st->scale_exp), rest);
   LBM_CUDA_TRY(cudaGetLastError());
@@ -281,7 +340,9 @@ int launch_get(const lbm_state* st, double* f) {
     const int rc = batch_relayout_pdfs(st, st->cur, st->cur ^ 1, true);
     if (rc != LBM_OK) return rc;
   }
-  get_pdfs_kernel<PREC><<<row_grid(st->sp->n), 256, 0, st->sp->stream>>>(
+  const auto kernel = st->sp->n <= kRowThreads * kRowBlocks ? get_pdfs_kernel<PREC, 1>
+                                                            : get_pdfs_kernel<PREC, kRowUnroll>;
+  kernel<<<row_grid(st->sp->n), kRowThreads, 0, st->sp->stream>>>(
       (const typename Form<PREC>::S*)st->buf[grouped ? st->cur ^ 1 : st->cur], f,
       (int32_t)st->sp->n, (int32_t)st->sp->ld, std::ldexp(1.0, -st->scale_exp));
   LBM_CUDA_TRY(cudaGetLastError());
