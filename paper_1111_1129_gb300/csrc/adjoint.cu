@@ -38,7 +38,7 @@
 // 76 + 76 lambda, 16 dJ/dalpha, 4 alpha; none of the 16 where dJ/dalpha is not
 // asked for) against 320 with g_t pulled from 19 rows through 32-bit links,
 // FP64 storage 398 against 560.  Damped 128^3 bed (1.03 M cells), against that
-// version: 200 steps and their gradient 26.6 -> 17.3 ms in FP32 shifted;
+// version: 200 steps and their gradient 26.6 -> 16.8 ms in FP32 shifted;
 // reverse pass of 2000 steps (a quarter of them kept) 178 -> 133 ms in FP32
 // shifted, 373 -> 302 in FP64 storage, 1,294 -> 1,031 in IEEE FP64, which is
 // bound by its arithmetic and no longer forms u a second time.
@@ -207,11 +207,75 @@ __device__ __forceinline__ void pull_adjoint(const T* __restrict__ lam_in, const
   for (int q = 1; q < 19; ++q) lf[opp(q)] = ld_nc(lam_in + idx[q - 1]);
 }
 
+// The reverse step of one cell in FP32 arithmetic: lf the pulled adjoints, out
+// the new ones in reversed rows, red its terms of dJ/dF.  Returns its term of
+// dJ/dalpha.
+template <class C, bool DAMPED>
+__device__ __forceinline__ C reverse_cell(const C lf[19], const C u[3], C al, const AdjCoef<C>& a,
+                                          C out[19], C red[4]) {
+  const C s = DAMPED ? C(1) / (C(1) + C(0.5) * al) : C(1);
+  C S[9], D[9];
+#pragma unroll
+  for (int p = 0; p < 9; ++p) {
+    S[p] = lf[2 * p + 1] + lf[2 * p + 2];
+    D[p] = lf[2 * p + 1] - lf[2 * p + 2];
+  }
+  // weighted moments of the adjoint
+  const C w0 = C(1.0 / 3.0), w1 = C(1.0 / 18.0), w2 = C(1.0 / 36.0);
+  const C M0 = w0 * lf[0] + w1 * (S[0] + S[1] + S[2]) +
+               w2 * (((S[3] + S[4]) + (S[5] + S[6])) + (S[7] + S[8]));
+  const C M1x = w1 * D[0] + w2 * ((D[3] + D[4]) + (D[5] + D[6]));
+  const C M1y = w1 * D[1] + w2 * ((D[3] - D[4]) + (D[7] + D[8]));
+  const C M1z = w1 * D[2] + w2 * ((D[5] - D[6]) + (D[7] - D[8]));
+  const C Mxx = w1 * S[0] + w2 * ((S[3] + S[4]) + (S[5] + S[6]));
+  const C Myy = w1 * S[1] + w2 * ((S[3] + S[4]) + (S[7] + S[8]));
+  const C Mzz = w1 * S[2] + w2 * ((S[5] + S[6]) + (S[7] + S[8]));
+  const C Mxy = w2 * (S[3] - S[4]);
+  const C Mxz = w2 * (S[5] - S[6]);
+  const C Myz = w2 * (S[7] - S[8]);
+  const C nine_wp = C(9) * a.wp, three_wp_m0 = C(3) * a.wp * M0;
+  const C beta = C(3) * (a.wm - al * a.src);
+  // G = nine_wp (M2 u) - three_wp_m0 u + beta M1, each rounding written out:
+  // left to the compiler, the sums contract differently from one
+  // instantiation of this kernel to the next
+  const auto G = [&](C q, C uj, C m1) {
+    return __fmaf_rn(beta, m1, __fmaf_rn(nine_wp, q, -__fmul_rn(three_wp_m0, uj)));
+  };
+  const C Gx = G(__fmaf_rn(Mxz, u[2], __fmaf_rn(Mxx, u[0], __fmul_rn(Mxy, u[1]))), u[0], M1x);
+  const C Gy = G(__fmaf_rn(Myz, u[2], __fmaf_rn(Myy, u[1], __fmul_rn(Mxy, u[0]))), u[1], M1y);
+  const C Gz = G(__fmaf_rn(Mzz, u[2], __fmaf_rn(Mxz, u[0], __fmul_rn(Myz, u[1]))), u[2], M1z);
+  const C base = a.wp * M0;
+  out[0] = a.one_m_wp * lf[0] + base;
+#define LBM_ADJ_PAIR(P, CG)                                                    \
+  {                                                                            \
+    const C sg_ = s * (CG);                                                    \
+    out[2 * P + 2] = a.k1 * lf[2 * P + 1] + a.k2 * lf[2 * P + 2] + base + sg_; \
+    out[2 * P + 1] = a.k1 * lf[2 * P + 2] + a.k2 * lf[2 * P + 1] + base - sg_; \
+  }
+  LBM_ADJ_PAIR(0, Gx)
+  LBM_ADJ_PAIR(1, Gy)
+  LBM_ADJ_PAIR(2, Gz)
+  LBM_ADJ_PAIR(3, Gx + Gy)
+  LBM_ADJ_PAIR(4, Gx - Gy)
+  LBM_ADJ_PAIR(5, Gx + Gz)
+  LBM_ADJ_PAIR(6, Gx - Gz)
+  LBM_ADJ_PAIR(7, Gy + Gz)
+  LBM_ADJ_PAIR(8, Gy - Gz)
+#undef LBM_ADJ_PAIR
+  const C hs = C(0.5) * s, three_src = C(3) * a.src;
+  red[0] = hs * Gx + three_src * M1x;
+  red[1] = hs * Gy + three_src * M1y;
+  red[2] = hs * Gz + three_src * M1z;
+  const C Gu = Gx * u[0] + Gy * u[1] + Gz * u[2];
+  const C M1u = M1x * u[0] + M1y * u[1] + M1z * u[2];
+  return -hs * Gu - three_src * M1u;
+}
+
 // One reverse step t: lam_f_t = S^T lam_g_{t+1} (pulled), then
 // lam_g_t = C'(g_t)^T lam_f_t with the velocity u of that collision, rows of
 // ld.  dalpha may be null (dJ/dalpha not wanted).
 // FP32 at 5 resident blocks (48 registers): 200 steps and their gradient on the
-// damped 128^3 bed 17.3 ms, 17.8 at 4 and 17.7 at 6.
+// damped 128^3 bed 17.3 ms, 17.8 at 4 and 17.7 at 6, when it served that list.
 #ifndef LBM_ADJ_MIN_BLOCKS
 #define LBM_ADJ_MIN_BLOCKS 5
 #endif
@@ -293,58 +357,102 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(C) == 4 ? LBM_ADJ_MIN_BL
       const C M1u = M1x * u[0] + M1y * u[1] + M1z * u[2];
       if (dalpha) dalpha[i] += (double)(-hs * Gu - a.src12 * M1u);
     } else {
-      // weighted moments of the adjoint
-      const C w0 = C(1.0 / 3.0), w1 = C(1.0 / 18.0), w2 = C(1.0 / 36.0);
-      const C M0 = w0 * lf[0] + w1 * (S[0] + S[1] + S[2]) +
-                   w2 * (((S[3] + S[4]) + (S[5] + S[6])) + (S[7] + S[8]));
-      const C M1x = w1 * D[0] + w2 * ((D[3] + D[4]) + (D[5] + D[6]));
-      const C M1y = w1 * D[1] + w2 * ((D[3] - D[4]) + (D[7] + D[8]));
-      const C M1z = w1 * D[2] + w2 * ((D[5] - D[6]) + (D[7] - D[8]));
-      const C Mxx = w1 * S[0] + w2 * ((S[3] + S[4]) + (S[5] + S[6]));
-      const C Myy = w1 * S[1] + w2 * ((S[3] + S[4]) + (S[7] + S[8]));
-      const C Mzz = w1 * S[2] + w2 * ((S[5] + S[6]) + (S[7] + S[8]));
-      const C Mxy = w2 * (S[3] - S[4]);
-      const C Mxz = w2 * (S[5] - S[6]);
-      const C Myz = w2 * (S[7] - S[8]);
-      const C nine_wp = C(9) * a.wp, three_wp_m0 = C(3) * a.wp * M0;
-      const C beta = C(3) * (a.wm - al * a.src);
-      // G = nine_wp (M2 u) - three_wp_m0 u + beta M1, each rounding written out:
-      // left to the compiler, the sums contract differently from one
-      // instantiation of this kernel to the next
-      const auto G = [&](C q, C uj, C m1) {
-        return __fmaf_rn(beta, m1, __fmaf_rn(nine_wp, q, -__fmul_rn(three_wp_m0, uj)));
-      };
-      const C Gx = G(__fmaf_rn(Mxz, u[2], __fmaf_rn(Mxx, u[0], __fmul_rn(Mxy, u[1]))), u[0], M1x);
-      const C Gy = G(__fmaf_rn(Myz, u[2], __fmaf_rn(Myy, u[1], __fmul_rn(Mxy, u[0]))), u[1], M1y);
-      const C Gz = G(__fmaf_rn(Mzz, u[2], __fmaf_rn(Mxz, u[0], __fmul_rn(Myz, u[1]))), u[2], M1z);
-      const C base = a.wp * M0;
-      lam_out[i] = a.one_m_wp * lf[0] + base;
-#define LBM_ADJ_PAIR(P, CG)                                                    \
-  {                                                                            \
-    const C sg_ = s * (CG);                                                    \
-    lam_out[(2 * P + 2) * ld + i] = a.k1 * lf[2 * P + 1] + a.k2 * lf[2 * P + 2] + base + sg_; \
-    lam_out[(2 * P + 1) * ld + i] = a.k1 * lf[2 * P + 2] + a.k2 * lf[2 * P + 1] + base - sg_; \
-  }
-      LBM_ADJ_PAIR(0, Gx)
-      LBM_ADJ_PAIR(1, Gy)
-      LBM_ADJ_PAIR(2, Gz)
-      LBM_ADJ_PAIR(3, Gx + Gy)
-      LBM_ADJ_PAIR(4, Gx - Gy)
-      LBM_ADJ_PAIR(5, Gx + Gz)
-      LBM_ADJ_PAIR(6, Gx - Gz)
-      LBM_ADJ_PAIR(7, Gy + Gz)
-      LBM_ADJ_PAIR(8, Gy - Gz)
-#undef LBM_ADJ_PAIR
-      const C hs = C(0.5) * s, three_src = C(3) * a.src;
-      red[0] = hs * Gx + three_src * M1x;
-      red[1] = hs * Gy + three_src * M1y;
-      red[2] = hs * Gz + three_src * M1z;
-      const C Gu = Gx * u[0] + Gy * u[1] + Gz * u[2];
-      const C M1u = M1x * u[0] + M1y * u[1] + M1z * u[2];
-      if (dalpha) dalpha[i] += (double)(-hs * Gu - three_src * M1u);
+      C out[19];
+      const C da = reverse_cell<C, DAMPED>(lf, u, al, a, out, red);
+#pragma unroll
+      for (int q = 0; q < 19; ++q) lam_out[q * ld + i] = out[q];
+      if (dalpha) dalpha[i] += (double)da;
     }
   }
   block_accumulate4(red, part + z + 4 * (int64_t)blockIdx.x, false);
+}
+
+// The same for lists with short links, two adjacent cells a thread as in
+// sweep_pair32_kernel: a warp takes one tile of links, a block of 128 threads
+// the 256 cells of a block above.  Its sums are formed in the same order: the
+// halves of a warp are the two warps above, and the last level of their tree
+// adds a thread's two cells.  Bound by latency and bytes (65% of the DRAM rate
+// in a launch of 40 us, 24 warps per SM); with 18 instead of 36 link loads for
+// two cells and twice the pulls in flight per thread, 200 steps and their
+// gradient on the damped 128^3 bed took 17.39 -> 16.83 ms, 40 steps on a
+// 151x141x201 bed 6.33 -> 6.04, 100 undamped steps of 128^3 7.62 -> 7.45.
+// Damped at 6 blocks per SM (80 registers), 17.1 ms at 5 and 17.9 at 7;
+// undamped at 5 (7.92 at 6, which spills).  Links loaded before the wait for
+// the previous step: 17.0.
+#ifndef LBM_ADJ_PAIR_MIN_BLOCKS
+#define LBM_ADJ_PAIR_MIN_BLOCKS 6
+#endif
+template <bool DAMPED>
+__global__ void __launch_bounds__(kSweepThreads / 2, DAMPED ? LBM_ADJ_PAIR_MIN_BLOCKS : 5)
+    adjoint_pair_kernel(const float* __restrict__ u_in, Links links, int32_t n, int32_t ld,
+                        AdjCoef<float> a, const float* __restrict__ alpha,
+                        const float* __restrict__ lam_in, float* __restrict__ lam_out,
+                        double* __restrict__ part, double* __restrict__ dalpha) {
+  const int32_t z = prior_step_done();  // as in adjoint_seed_kernel
+  const int32_t i = 2 * (int32_t)(blockIdx.x * (kSweepThreads / 2) + threadIdx.x) + z;
+  const bool two = i + 1 < n;
+  float r[2][4] = {};
+  if (i < ld) {   // whole warps
+    uint32_t word[18];
+    int32_t entry;
+    load_pair_links(links, ld, i, word, entry);
+    float lf[2][19];
+    if (i < n) lf[0][0] = ld_nc(lam_in + i);
+    if (two) lf[1][0] = ld_nc(lam_in + i + 1);
+#pragma unroll
+    for (int q = 1; q < 19; ++q) {
+      const int32_t m0 = short_slot(q, ld, entry, word[q - 1]);
+      const int32_t m1 = short_slot(q, ld, entry, word[q - 1] >> 16);
+      if (i < n) lf[0][opp(q)] = ld_nc(lam_in + m0);
+      if (two) lf[1][opp(q)] = ld_nc(lam_in + m1);
+    }
+    if (i < n) {
+      // past the end of an odd list: the padding of the rows of ld
+      float2 u[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) u[j] = ld_nc(reinterpret_cast<const float2*>(u_in + j * ld + i));
+      const float al0 = DAMPED ? ld_nc(alpha + i) : 0.f;
+      const float al1 = DAMPED && two ? ld_nc(alpha + i + 1) : 0.f;
+      float out[19];
+      const float u0[3] = {u[0].x, u[1].x, u[2].x}, u1[3] = {u[0].y, u[1].y, u[2].y};
+      const float d0 = reverse_cell<float, DAMPED>(lf[0], u0, al0, a, out, r[0]);
+      if (two) {
+        float out1[19];
+        const float d1 = reverse_cell<float, DAMPED>(lf[1], u1, al1, a, out1, r[1]);
+#pragma unroll
+        for (int q = 0; q < 19; ++q)
+          *reinterpret_cast<float2*>(lam_out + q * ld + i) = make_float2(out[q], out1[q]);
+        if (dalpha) {
+          double2* at = reinterpret_cast<double2*>(dalpha + i);
+          const double2 v = *at;
+          *at = make_double2(v.x + (double)d0, v.y + (double)d1);
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < 19; ++q) lam_out[q * ld + i] = out[q];
+        if (dalpha) dalpha[i] += (double)d0;
+      }
+    }
+  }
+  // block_accumulate4 of 256 cells
+  __shared__ double sm[kSweepThreads / 32][4];
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      r[0][j] += __shfl_down_sync(0xffffffffu, r[0][j], o);
+      r[1][j] += __shfl_down_sync(0xffffffffu, r[1][j], o);
+    }
+  if ((threadIdx.x & 15) == 0)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) sm[threadIdx.x >> 4][j] = (double)(r[0][j] + r[1][j]);
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kSweepThreads / 32; ++w) s += sm[w][threadIdx.x];
+    part[z + 4 * (int64_t)blockIdx.x + threadIdx.x] += s;
+  }
 }
 
 // ---- FP64-storage adjoint in double-single arithmetic --------------------------
@@ -595,10 +703,14 @@ struct Runner {
   E* lam(int i) const { return (E*)ad->lam[i]; }
 
   template <class... P, class... A>
-  void launch(void (*kernel)(P...), A... args) {
-    const cudaError_t e = launch_sweep(kernel, grid, stream, kChain && chained, args...);
+  void launch_threads(void (*kernel)(P...), unsigned threads, A... args) {
+    const cudaError_t e = launch_chained(kernel, grid, threads, stream, kChain && chained, args...);
     if (err == cudaSuccess) err = e;
     chained = true;
+  }
+  template <class... P, class... A>
+  void launch(void (*kernel)(P...), A... args) {
+    launch_threads(kernel, (unsigned)kSweepThreads, args...);
   }
   void step(const void* src, void* dst, E* u_out) {
     const cudaError_t e = launch_plain_step(st, src, dst, u_out, ad->wp, ad->wm, ad->F, stream,
@@ -627,6 +739,9 @@ struct Runner {
     if constexpr (PREC == LBM_F64X)
       launch(adjoint_step_ds_kernel<DA, SH>, u_in, links, n, ld, ads, alpha,
              (const int64_t*)st->alpha_fx, (const float2*)lam(in), lam(in ^ 1), ad->part, dalpha);
+    else if constexpr (SH && sizeof(C) == 4)
+      launch_threads(adjoint_pair_kernel<DA>, (unsigned)kSweepThreads / 2, u_in, links, n, ld, a, alpha,
+                     (const C*)lam(in), lam(in ^ 1), ad->part, dalpha);
     else
       launch(adjoint_step_kernel<C, DA, SH>, u_in, links, n, ld, a, alpha, (const C*)lam(in),
              lam(in ^ 1), ad->part, dalpha);

@@ -93,3 +93,40 @@ def test_list_with_short_links_matches_oracle(precision, damped):
     adj.close()
     st.close()
     lat.close()
+
+
+@pytest.mark.parametrize("damped", [False, True])
+@pytest.mark.parametrize("odd", [False, True])
+@pytest.mark.parametrize("precision", ["f32s", "f16s"])
+def test_two_cells_a_thread_match_one(precision, odd, damped):
+    """Five copies of a periodic box, long enough for short links and the reverse
+    step of two cells a thread, against one copy with a cell a thread: the same
+    mean velocity, and each cell's gradient a fifth.  The seeds 1/N round
+    differently; a value takes ~10 roundings of 2^-24 in each of 4 steps, which
+    1e-5 of the norm covers."""
+    flags, alpha, f0 = _random((45, 44, 43), 11, 1e-3)
+    fluid = np.argwhere(flags == 0)
+    if (len(fluid) % 2 == 1) != odd:
+        flags[tuple(fluid[777])] = 1
+        f0 = f0 * (flags == 0)
+    got = []
+    for copies in (1, 5):
+        tile = lambda a: np.concatenate([a] * copies, axis=-3)
+        lat = SparseLattice(torch.from_numpy(tile(flags)).cuda(), "lex", periodic=7)
+        st = _state(lat, precision, tile(f0), tile(alpha) if damped else None)
+        adj = Adjoint(st, 4)
+        J = adj.forward(WP, WM, F, 0)
+        dF, da, _ = adj.backward(want_alpha=True)
+        got.append((J, np.array(dF), da.cpu().numpy() * copies, lat.n))
+        adj.close()
+        st.close()
+        lat.close()
+    (J1, dF1, da1, n1), (J5, dF5, da5, n5) = got
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert n1 % 2 == odd and n1 <= 2 * 4 * 256 * sms < n5 == 5 * n1
+
+    def rel(a, b):
+        return np.linalg.norm(a - b) / np.linalg.norm(b)
+    assert abs(J5 - J1) <= 1e-5 * abs(J1)
+    assert rel(dF5, dF1) < 1e-5
+    assert rel(da5.reshape(5, n1), da1[None].repeat(5, 0)) < 1e-5
