@@ -64,6 +64,7 @@ struct Coef {
   C F[3], hF[3];   // F, F / 2
   C bF1[3];        // b1 F (used without damping)
   C scale, inv_scale;
+  C c15;           // 1.5 (scaled() changes it)
   C rest;          // FP64 collision: (1 - (1 - w+)) / (w+ / 18) - 12 in working precision, ~6
 };
 
@@ -87,10 +88,27 @@ Coef<C> make_coef(double wp, double wm, const double F[3], int scale_exp) {
   }
   k.scale = (C)std::ldexp(1.0, scale_exp);
   k.inv_scale = (C)std::ldexp(1.0, -scale_exp);
+  k.c15 = (C)1.5;
   // the rest population takes what the rounded 1 - w+ and w+/18 of the other
   // 18 leave of a cell's mass: no drift from the rounding of constants
   const double gone = 1.0 - (1.0 - wp), w1 = wp / 18.0, q = gone / w1;
   k.rest = (C)((q - 12.0) + std::fma(-q, w1, gone) / w1);
+  return k;
+}
+
+// The coefficients of a collision of values times `scale`, exact powers of two:
+// linear terms keep theirs, the force takes the scale and the quadratic terms
+// its inverse.
+template <class C>
+Coef<C> scaled(Coef<C> k) {
+  for (int d = 0; d < 3; ++d) {
+    k.F[d] *= k.scale;
+    k.hF[d] *= k.scale;
+    k.bF1[d] *= k.scale;
+  }
+  k.k1 *= k.inv_scale;
+  k.k2 *= k.inv_scale;
+  k.c15 *= k.inv_scale;
   return k;
 }
 
@@ -241,7 +259,8 @@ __device__ __forceinline__ void collide_f64(double g[19], const Coef<double>& k,
 }
 
 // g[19] in: pulled PDFs (or deviations); out: post-collision values.
-template <class C, bool DAMPED>
+// SCALED: the values, rho and u are times k.scale, with coefficients scaled().
+template <class C, bool DAMPED, bool SCALED = false>
 __device__ __forceinline__ void collide(C g[19], const Coef<C>& k, C alpha, C& rho_out,
                                         C u_out[3]) {
   if constexpr (sizeof(C) == 8) {
@@ -278,7 +297,7 @@ __device__ __forceinline__ void collide(C g[19], const Coef<C>& k, C alpha, C& r
     Vz = k.a1 * uz + k.bF1[2];
   }
   const C usq = ux * ux + uy * uy + uz * uz;
-  const C rp = rho - C(1.5) * usq;
+  const C rp = rho - (SCALED ? k.c15 : C(1.5)) * usq;
   const C R1 = k.w1p * rp, R2 = C(0.5) * R1;
   g[0] = k.one_m_wp * g[0] + k.w0p * rp;
 #define LBM_PAIR(P, CU, CV, R, K, HALF)                    \
@@ -601,14 +620,22 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_launch_min_blocks<PREC, R
 }
 
 template <int PREC>
-__device__ __forceinline__ float bits_to_c(uint32_t h, float inv_scale) {
-  if constexpr (PREC == LBM_F16S) return __half2float(__ushort_as_half((unsigned short)h)) * inv_scale;
-  else return __bfloat162float(__ushort_as_bfloat16((unsigned short)h)) * inv_scale;
+__device__ __forceinline__ float low_value(uint32_t pair) {
+  if constexpr (PREC == LBM_F16S) return __half2float(__ushort_as_half((unsigned short)pair));
+  else return __uint_as_float(pair << 16);
 }
 template <int PREC>
-__device__ __forceinline__ uint32_t c_to_bits(float v, float scale) {
-  if constexpr (PREC == LBM_F16S) return __half_as_ushort(__float2half_rn(v * scale));
-  else return __bfloat16_as_ushort(__float2bfloat16_rn(v * scale));
+__device__ __forceinline__ float high_value(uint32_t pair) {
+  if constexpr (PREC == LBM_F16S) return __half2float(__ushort_as_half((unsigned short)(pair >> 16)));
+  else return __uint_as_float(pair & 0xffff0000u);
+}
+// Two values rounded to the form, packed (one instruction).
+template <int PREC>
+__device__ __forceinline__ uint32_t pack_values(float low, float high) {
+  uint32_t r;
+  if constexpr (PREC == LBM_F16S) asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(high), "f"(low));
+  else asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(high), "f"(low));
+  return r;
 }
 
 // ---- two adjacent cells per thread ------------------------------------------
@@ -618,15 +645,18 @@ __device__ __forceinline__ uint32_t c_to_bits(float v, float scale) {
 // results (every row is aligned: the row stride is a multiple of kRowAlign);
 // the pulls stay scalar, back to back, so that each pair lands on the same
 // sectors and L1 merges them.  The per-cell arithmetic is that of
-// sweep_kernel, so results are bit-identical to it.
+// sweep_kernel, up to exact powers of two, so results are bit-identical to it.
 //
 // What bounds them: DRAM bytes in FP32 (190 per update, 38 of them links), the
-// latency of the two dependent round trips (codes, then pulls) in the 16-bit
-// forms.  1024x256x256 bed, MFLUP/s, lexicographic / 8^3 blocked order:
+// latency of the two dependent round trips (codes, then pulls) and half of the
+// issue slots in the 16-bit forms.  1024x256x256 bed, MFLUP/s, lexicographic /
+// 8^3 blocked order:
 //   FP32S  one cell, 32-bit links 31,444 / 30,249; one cell, short links
 //          32,380 / 31,396; pair 36,746 / 35,079 (1.05 of the copy rate)
-//   FP16S  pair, 32-bit links 45,648 / 43,751; pair, short links
-//          51,409 / 49,378 (0.88)
+//   FP16S  pair, 32-bit links 45,648 / 43,751; short links 51,409 / 49,378;
+//          arithmetic on the stored values (coefficients scaled(), no product
+//          with the scale) and both cells rounded and packed by one
+//          instruction 52,941 / 50,533 (0.91)
 // Launch shapes: FP32 in 128-thread blocks at 6 per SM (80 registers); 7 per
 // SM 36,786 / 35,061, 5 36,457 / 34,880, 256 threads x 3 36,596 and x 4
 // (64 registers, spills) 34,956 in lexicographic order.  16-bit forms in
@@ -697,31 +727,29 @@ __global__ void __launch_bounds__(kPairThreads, LBM_PAIR_MIN_BLOCKS)
     const uint32_t hi = two ? (uint32_t)ld_nc(src16 + b[q]) : 0u;
     g[q + 1] = lo | (hi << 16);
   }
-  uint32_t out[19];
+  // the arithmetic is that of the stored values, times k.scale
+  float v0[19], v1[19], rho, u0[3], u1[3];
 #pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    if (c == 0 || two) {
-      float v[19], rho, u[3];
-#pragma unroll
-      for (int q = 0; q < 19; ++q) v[q] = bits_to_c<PREC>(c ? g[q] >> 16 : g[q] & 0xffffu, k.inv_scale);
-      collide<float, DAMPED>(v, k, DAMPED ? ld_nc(alpha + i + c) : 0.f, rho, u);
-#pragma unroll
-      for (int q = 0; q < 19; ++q) {
-        const uint32_t h = c_to_bits<PREC>(v[q], k.scale);
-        out[q] = c ? out[q] | (h << 16) : h;
-      }
-      if constexpr (KEEP_U)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) st_cs(u_out + j * ld + i + c, u[j]);
-    }
+  for (int q = 0; q < 19; ++q) {
+    v0[q] = low_value<PREC>(g[q]);
+    v1[q] = high_value<PREC>(g[q]);
   }
+  collide<float, DAMPED, true>(v0, k, DAMPED ? ld_nc(alpha + i) : 0.f, rho, u0);
+  if (two) collide<float, DAMPED, true>(v1, k, DAMPED ? ld_nc(alpha + i + 1) : 0.f, rho, u1);
   unsigned short* dst16 = reinterpret_cast<unsigned short*>(dst);
 #pragma unroll
   for (int q = 0; q < 19; ++q) {
     const int32_t e = q * ld + i;   // even: one 4-byte store of the pair
-    if (two) asm volatile("st.global.cs.u32 [%0], %1;" ::"l"(dst16 + e), "r"(out[q]) : "memory");
-    else st_cs(dst16 + e, (unsigned short)(out[q] & 0xffffu));
+    const uint32_t out = pack_values<PREC>(v0[q], v1[q]);
+    if (two) asm volatile("st.global.cs.u32 [%0], %1;" ::"l"(dst16 + e), "r"(out) : "memory");
+    else st_cs(dst16 + e, (unsigned short)(out & 0xffffu));
   }
+  if constexpr (KEEP_U)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      st_cs(u_out + j * ld + i, u0[j] * k.inv_scale);
+      if (two) st_cs(u_out + j * ld + i + 1, u1[j] * k.inv_scale);
+    }
 }
 
 // The same for the FP32 forms.

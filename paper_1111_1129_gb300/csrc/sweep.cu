@@ -214,7 +214,8 @@ cudaError_t launch_step(const lbm_state* st, const typename Form<PREC>::S* src,
   };
   const auto pair = [&](auto* kernel, int64_t threads) {
     return launch_chained(kernel, (unsigned)((n + 2 * threads - 1) / (2 * threads)),
-                          (unsigned)threads, stream, chained, src, dst, links, n, ld, k, alpha,
+                          (unsigned)threads, stream, chained, src, dst, links, n, ld,
+                          compute_bytes(PREC) == storage_bytes(PREC) ? k : scaled(k), alpha,
                           u_out);
   };
   if (reduce) return sweep(sweep_kernel<PREC, DAMPED, kWarpSums, SHORT>);
