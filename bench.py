@@ -46,14 +46,25 @@ BYTES_PER_LUP = {"f64": 19 * 8 * 2 + 18 * 4, "f64x": 19 * 8 * 2 + 18 * 4,
                  "f32": 19 * 4 * 2 + 18 * 4,
                  "f32s": 19 * 4 * 2 + 18 * 4, "f16s": 19 * 2 * 2 + 18 * 4,
                  "bf16s": 19 * 2 * 2 + 18 * 4}
+# Lists above two waves of the sweep (2 x 4 x 256 cells per SM) keep their links
+# in 18 codes of 2 bytes and 32 page entries per 64 cells: 38 bytes for 72.
+SHORT_LINK_SAVING = 18 * 4 - (18 * 2 + 32 * 4 / 64)
+
+
+def _bytes_per_lup(prec, n):
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return BYTES_PER_LUP[prec] - (SHORT_LINK_SAVING if n > 2 * 4 * 256 * sms else 0)
+
+
 # DRAM bytes (read + write) per fluid update of one sweep launch, measured by
 # ncu (dram__bytes_read.sum + dram__bytes_write.sum of one launch, after
 # three warm-up steps) per (workload, form, ordering).  The roofline's
 # `traffic` multiplies them by the benchmark's cells.  Drop an entry when its
 # kernel changes.
 MEASURED_DRAM_BYTES_PER_LUP = {
-    ("large", "f64x", "lex"): 379.9, ("large", "f32s", "lex"): 223.4,
-    ("large", "f16s", "lex"): 147.2,
+    ("large", "f64x", "lex"): 344.0, ("large", "f32s", "lex"): 189.0,
+    ("large", "f16s", "lex"): 113.0,
 }
 STORAGE = {"f64": "f64", "f64x": "f64", "f32": "f32", "f32s": "f32 (f - w)",
            "f16s": "f16 ((f - w) 2^k)", "bf16s": "bf16 ((f - w) 2^k)"}
@@ -352,8 +363,8 @@ def run_ours(args):
                          f"full-array oracle ({dt:.1f} s)"}
     lat.close()
     peak, peak_kind = _peaks()
-    bpl = BYTES_PER_LUP[args.precision]
-    ws = (2 * 19 * (bpl - 72) / 38 + 72) * n   # two PDF grids + adjacency, bytes
+    bpl = _bytes_per_lup(args.precision, n)
+    ws = bpl * n   # two PDF grids + links, bytes
     achieved = bpl * n / (launch_ms * 1e-3) / 1e9
     line = {
         "metric": "MFLUP/s", "value": value, "unit": "MFLUP/s", "n_gpus": world,
@@ -377,9 +388,11 @@ def run_ours(args):
                                  in MEASURED_DRAM_BYTES_PER_LUP else None),
                      "bytes_per_lup": bpl, "peak_kind": peak_kind,
                      "kernel": "sweep_fx_kernel" if args.precision == "f64x"
-                     else (f"sweep_pair_kernel<{args.precision}>"
-                           if args.precision in ("f16s", "bf16s") else
-                           f"sweep_kernel<{args.precision}>")},
+                     else f"sweep_kernel<{args.precision}>"
+                     if args.precision == "f64" or bpl == BYTES_PER_LUP[args.precision]
+                     else f"sweep_pair32_kernel<{args.precision}>"
+                     if args.precision in ("f32", "f32s")
+                     else f"sweep_pair_kernel<{args.precision}>"},
         "e2e": {"value": e2e_value, "unit": "MFLUP/s",
                 "h2d_bytes_per_step": (bed.flags.nbytes + 24) / args.steps,
                 "d2h_bytes_per_step": 32 / args.steps,
@@ -388,7 +401,8 @@ def run_ours(args):
                          "allocator (lbm_set_allocator), warm from the device-timed run; median "
                          "of 3 independent calls",
                 "samples_mflups": [n * args.steps / t / 1e6 for t in e2e_times]},
-        "gpu_launches": args.steps + 2,
+        # the sweeps and the sums, which take two launches above 2^20 cells
+        "gpu_launches": args.steps + (2 if n > 1 << 20 else 1),
         "clocks": clocks.summary(),
         "result": {"mass": mass, "flux": flux, "e2e_flux": e2e_flux},
     }
@@ -828,7 +842,7 @@ def run_seed_study(args):
             torch.cuda.synchronize()
             rate = lat.n * args.extra_steps / (e0.elapsed_time(e1) * 1e-3) / 1e6
             row[f"{prec}_mflups"] = rate
-            row[f"{prec}_frac"] = rate * 1e6 * BYTES_PER_LUP[prec] / 1e9 / peak
+            row[f"{prec}_frac"] = rate * 1e6 * _bytes_per_lup(prec, lat.n) / 1e9 / peak
             st.close()
         rows.append(row)
         lat.close()

@@ -25,8 +25,10 @@ std::atomic<int64_t> g_live{0};
 // time of assembling a large lattice (1024x256x256 bed with its outputs 11.9
 // ms, 2.8 ms with the pool).  Memory beyond that goes back to the device when the
 // stream is next synchronised; all of it when an allocation of the library
-// fails or lbm_set_allocator is called.  The driver orders the reuse of a block
-// across streams, and the calls are safe from several threads.
+// fails or lbm_set_allocator is called, and the driver takes it for a cudaMalloc
+// of the process that needs it (with 4.0 GB idle, one of the free memory and
+// 2.0 GB more succeeded).  The driver orders the reuse of a block across streams,
+// and the calls are safe from several threads.
 constexpr int kMaxDevices = 64;
 std::mutex g_pool_mutex;
 cudaMemPool_t g_pool[kMaxDevices] = {};

@@ -831,7 +831,7 @@ __device__ __forceinline__ void tree_sum_1024(double (*sm)[4]) {
   }
 }
 
-// The flux sums of a step from its per-warp slots, in one launch.  Thread b
+// The flux sums of a step from its per-warp slots.  Thread b
 // forms block b's value (its kWarpsPerBlock slots in slot order, the value
 // store_block_sums forms inside a block); each 256-thread CTA adds its 256
 // block values by a fixed tree into groups[4 g + j]; and the last CTA to arrive
@@ -839,8 +839,12 @@ __device__ __forceinline__ void tree_sum_1024(double (*sm)[4]) {
 // sums to `out`, which may be pinned host memory, so that nothing is copied.
 // One 1024-thread block reading all block values had cost 0.15 ms per call on
 // the 1024x256x256 bed; two kernels and a copy cost a short call two launches.
-// *arrived counts the CTAs and wraps to 0.
-constexpr int kCollapseThreads = 256;
+// *arrived counts the CTAs and wraps to 0; null: the groups only, which
+// final_sum_kernel adds in a launch of its own.  One launch takes 25 us with the
+// host's wait up to 64 groups, two 27; at 1024 groups, where 1024 threads add
+// them faster, 72 and 66.  So lists above 16 groups (1,048,576 cells, steps of
+// 20 us and more) take two.
+constexpr int kCollapseThreads = 256, kOneLaunchGroups = 16;
 __global__ void __launch_bounds__(kCollapseThreads)
     flux_sums_kernel(const double* __restrict__ part, int64_t nblocks, double* groups,
                      unsigned* arrived, double* out) {
@@ -865,6 +869,7 @@ __global__ void __launch_bounds__(kCollapseThreads)
     __syncthreads();
   }
   if (threadIdx.x < 4) groups[4 * blockIdx.x + threadIdx.x] = sm[0][threadIdx.x];
+  if (!arrived) return;
   __threadfence();   // the group's value before the arrival
   __syncthreads();
   if (threadIdx.x == 0) last = atomicInc(arrived, gridDim.x - 1) == gridDim.x - 1;

@@ -697,8 +697,10 @@ extern "C" int lbm_reduce_flux(lbm_state* st, int32_t axis, double* mass_out, do
     // group sums after the warp slots (room for nblocks values of 4)
     double* groups = st->partials + 4 * kWarpsPerBlock * st->nblocks;
     const int64_t ngroups = (st->nblocks + kCollapseThreads - 1) / kCollapseThreads;
+    const bool one = ngroups <= kOneLaunchGroups;
     flux_sums_kernel<<<(unsigned)ngroups, kCollapseThreads, 0, stream>>>(
-        st->partials, st->nblocks, groups, st->arrived, st->red_host);
+        st->partials, st->nblocks, groups, one ? st->arrived : nullptr, st->red_host);
+    if (!one) final_sum_kernel<<<1, 1024, 0, stream>>>(groups, ngroups, st->red_host);
     LBM_CUDA_TRY(cudaGetLastError());
     const int rc = wait_event(st->done, stream, 0.0);
     if (rc != LBM_OK) return rc;
