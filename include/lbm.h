@@ -66,7 +66,8 @@ extern "C" {
 #define LBM_OK 0
 #define LBM_EINVAL (-1)      /* bad argument (null pointer, size, range) */
 #define LBM_EOVERFLOW (-2)   /* index space beyond int32: box >= 2^31 cells
-                                or 19*N >= 2^31 PDF slots */
+                                or 19*N >= 2^31 PDF slots; or an axis longer
+                                than an ordering's keys can hold */
 #define LBM_ECUDA (-3)       /* a CUDA runtime call failed */
 #define LBM_ENONFINITE (-4)  /* a reduction produced NaN or Inf */
 #define LBM_ETIMEOUT (-5)    /* queued work did not finish in the time limit */
@@ -115,7 +116,8 @@ typedef struct lbm_state lbm_state;
  * Numbering-scheme key I(x,y,z) of every box cell (Sec. 3, "Numbering
  * scheme": a unique, not necessarily contiguous index of all cells).
  * keys_dev: device uint64[nx*ny*nz] in box layout, written on `stream`.
- * Returns LBM_EINVAL for bad dims or ordering.
+ * Returns LBM_EINVAL for bad dims or ordering, LBM_EOVERFLOW for a curve with
+ * an axis above 2^21 cells (LBM_ORDER_MORTON2: 2^20).
  */
 int lbm_ordering_keys(const int32_t dims[3], lbm_ordering ord, uint64_t* keys_dev,
                       void* stream);

@@ -655,6 +655,12 @@ int make_key_space(const int32_t dims[3], const lbm_ordering& ord, bool clamp_bl
   s.nbz = (s.nz + s.bz - 1) / s.bz;
   s.hbits = 1;
   while ((1LL << s.hbits) < s.nx || (1LL << s.hbits) < s.ny || (1LL << s.hbits) < s.nz) ++s.hbits;
+  // curve keys keep this many bits of each coordinate (key_of); a longer axis
+  // would give several cells one key
+  const int32_t key_bits = ord.kind == LBM_ORDER_MORTON2 ? 20 : 21;
+  if (is_curve(ord.kind) && s.hbits > key_bits)
+    return fail(LBM_EOVERFLOW, "an axis of more than 2^%d cells exceeds the keys of this ordering",
+                (int)key_bits);
   if (ord.kind == LBM_ORDER_BLOCKED) {
     s.size = (uint64_t)(s.nbx * s.nby * s.nbz) * (uint64_t)(s.bx * s.by * s.bz);
   } else if (ord.kind == LBM_ORDER_HILBERT) {
