@@ -672,7 +672,9 @@ int make_key_space(const int32_t dims[3], const lbm_ordering& ord, bool clamp_bl
     // far corner holds the largest key
     s.size = key_of(s, s.nx - 1, s.ny - 1, s.nz - 1) + 1;
   }
-  if (ord.kind == LBM_ORDER_BLOCKED && s.size < (1ull << 31)) {
+  // for the walk, whose blocks are no larger than the box: literal blocks may
+  // span a key space of more than 64 bits, and size is then no measure of it
+  if (ord.kind == LBM_ORDER_BLOCKED && clamp_blocks && s.size < (1ull << 31)) {
     s.by_bsz = fixed_div((uint32_t)(s.bx * s.by * s.bz));
     s.by_bx = fixed_div((uint32_t)s.bx);
     s.by_bxy = fixed_div((uint32_t)(s.bx * s.by));

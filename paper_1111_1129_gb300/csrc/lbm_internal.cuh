@@ -91,7 +91,8 @@ struct KeySpace {
   // unit[a]: the key of the unit vector along axis a on that small curve.
   int32_t levels;
   uint32_t unit[3];
-  // Blocked order with a key space below 2^31: the divisors of blocked_cell.
+  // Blocked order as the assembly walks it, with a key space below 2^31: the
+  // divisors of blocked_cell.
   FixedDiv by_bsz, by_bx, by_bxy, by_nbx, by_nbxy;
 };
 

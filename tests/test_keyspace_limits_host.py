@@ -71,3 +71,20 @@ def test_curve_keys_are_not_cut(tool, kind, bits, axis, walk):
                           for b in range(bits))
     dims[axis] += 1
     assert tool(dims, kind, (1, 1, 1), walk)[0] == EOVERFLOW
+
+
+@pytest.mark.parametrize("dims,block", [((1, 1, 16), (2 ** 30, 2 ** 30, 4)),
+                                        ((1, 4, 16), (2 ** 30, 2, 2 ** 31 - 1)),
+                                        ((3, 1, 32), (2 ** 30, 2 ** 29, 8))])
+def test_blocks_far_beyond_the_box_have_keys(tool, dims, block):
+    """Keys keep the literal blocking factors, so their space may span more
+    than 64 bits although every key of the box fits."""
+    last = [d - 1 for d in dims]
+    blocks = [-(-d // b) for d, b in zip(dims, block)]
+    of = [c // b for c, b in zip(last, block)]
+    at = [c % b for c, b in zip(last, block)]
+    number = of[0] + blocks[0] * (of[1] + blocks[1] * of[2])
+    key = (number * block[0] * block[1] * block[2] +
+           at[0] + block[0] * (at[1] + block[1] * at[2]))
+    assert key < 2 ** 64
+    assert tool(dims, 1, block, False) == (OK, key)
