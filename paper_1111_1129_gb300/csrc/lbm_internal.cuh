@@ -453,6 +453,7 @@ struct StepGraph {
   cudaGraphExec_t exec[2];  // per parity of st->cur, or null
   double wp[2], wm[2], F[2][3];
   const void* alpha[2];
+  const int64_t* alpha_fx[2];   // an allocation of its own
 };
 
 // Launches a sweep on `stream` in blocks of kSweepThreads.  `chained` means

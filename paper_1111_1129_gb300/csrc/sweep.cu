@@ -393,7 +393,8 @@ int step_graph(lbm_state* st, double wp, double wm, const double F[3], cudaGraph
   StepGraph* g = st->graph;
   const int p = st->cur;
   if (g->exec[p] && g->wp[p] == wp && g->wm[p] == wm && g->F[p][0] == F[0] &&
-      g->F[p][1] == F[1] && g->F[p][2] == F[2] && g->alpha[p] == st->alpha) {
+      g->F[p][1] == F[1] && g->F[p][2] == F[2] && g->alpha[p] == st->alpha &&
+      g->alpha_fx[p] == st->alpha_fx) {
     *out = g->exec[p];
     return LBM_OK;
   }
@@ -421,6 +422,7 @@ int step_graph(lbm_state* st, double wp, double wm, const double F[3], cudaGraph
   g->wm[p] = wm;
   for (int d = 0; d < 3; ++d) g->F[p][d] = F[d];
   g->alpha[p] = st->alpha;
+  g->alpha_fx[p] = st->alpha_fx;
   *out = g->exec[p];
   return LBM_OK;
 }
