@@ -158,6 +158,8 @@ int lbm_build_sparse(const uint8_t* flags, const int32_t dims[3], lbm_ordering o
  * layout above; unless the steps' links are that array the first request builds it
  * (72 bytes per cell of device memory, one kernel on the handle's stream,
  * which the call then synchronises) and may fail with LBM_ENOMEM.
+ * lbm_free gives them back in the order of the handle's stream, for the next
+ * lattice to write: what reads them on another stream has to finish before.
  */
 int lbm_sparse_info(const lbm_sparse* sp, int64_t* n_fluid, const int32_t** cells_dev,
                     const int32_t** adj_dev, const int32_t** inv_dev);

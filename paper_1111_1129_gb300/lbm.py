@@ -118,6 +118,7 @@ class SparseLattice:
         self.ordering = ordering
         self.block = tuple(block)
         self.periodic = int(periodic)
+        self._reads = {}   # the last copy queued on each stream but the lattice's own
         self._handle = None
         self._handle = capi.lbm_build_sparse(
             flags.data_ptr(), self.dims,
@@ -131,20 +132,32 @@ class SparseLattice:
     def handle(self) -> int:
         return self._handle
 
+    def _copy(self, ptr: int, shape) -> torch.Tensor:
+        """Copy of int32 device memory of the handle, on the current stream.
+        The handle gives its memory back in the order of the lattice's own
+        stream, for the next lattice to write; so close() waits for the last
+        copy queued on any other."""
+        out = _borrow(ptr, shape, "<i4", torch.int32).clone()
+        here = torch.cuda.current_stream()
+        if (here.cuda_stream != self.stream.cuda_stream
+                and not torch.cuda.is_current_stream_capturing()):
+            self._reads[here.cuda_stream] = here.record_event()
+        return out
+
     def cells(self) -> torch.Tensor:
         """Copy of cells[N] (box index of each fluid cell, in order)."""
-        return _borrow(self._cells, (self.n,), "<i4", torch.int32).clone()
+        return self._copy(self._cells, (self.n,))
 
     def adjacency(self) -> torch.Tensor:
         """Copy of adj[18, N] (slot q N + m)."""
         if not self._adj:
             self._adj = capi.lbm_sparse_info(self._handle)[2]
-        return _borrow(self._adj, (18, self.n), "<i4", torch.int32).clone()
+        return self._copy(self._adj, (18, self.n))
 
     def inverse(self) -> torch.Tensor:
         """Copy of inv[nz, ny, nx] (fluid index or -1)."""
         nx, ny, nz = self.dims
-        return _borrow(self._inv, (nz, ny, nx), "<i4", torch.int32).clone()
+        return self._copy(self._inv, (nz, ny, nx))
 
     def gather(self, dense: torch.Tensor) -> torch.Tensor:
         """Box-layout field [..., nz, ny, nx] -> fluid order [..., N]."""
@@ -153,8 +166,12 @@ class SparseLattice:
 
     def close(self):
         if self._handle:
-            capi.lbm_free(self._handle)
-            self._handle = None
+            handle, self._handle = self._handle, None
+            try:
+                for copied in self._reads.values():
+                    copied.synchronize()
+            finally:
+                capi.lbm_free(handle)
 
     def __del__(self):
         try:
