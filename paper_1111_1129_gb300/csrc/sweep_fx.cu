@@ -359,8 +359,9 @@ __global__ void __launch_bounds__(kSweepThreads, LBM_FX_RED_MIN_BLOCKS)
     fast = fx_moments(b, k, S, D, drho, ux, uy, uz) &&
            fx_damp<DAMPED>(alpha_fx, n, i, k, ux, uy, uz, a1);
   }
-  fast ? fx_fixed_warp_sums(drho, ux, uy, uz, 1, partials + z)
-       : fx_fixed_warp_sums(0, 0, 0, 0, 0, partials + z);
+  // one call for the whole warp, whose lanes may take either path
+  fx_fixed_warp_sums(fast ? drho : 0, fast ? ux : 0, fast ? uy : 0, fast ? uz : 0, fast ? 1 : 0,
+                     partials + z);
   double red[4] = {0.0, 0.0, 0.0, 0.0};   // IEEE-path cells: rho, u
   if (live) {
     if (fast) {
