@@ -864,7 +864,7 @@ extern "C" int lbm_build_sparse(const uint8_t* flags, const int32_t dims[3], lbm
   // 17,853, FP16S 18,730 / 18,446; 221,119 cells FP64 storage 19,623 / 21,163,
   // FP32S 37,045 / 43,126, FP16S 36,547 / 44,828;
   // 413,546 cells FP64 storage 16,411 / 14,675, FP32S 43,166 / 38,031.
-  const bool brief = n > 2 * one_wave_cells();
+  const bool brief = n > small_list_cells();
   const auto alloc_wide = [&]() {   // they are the public links when ld == n
     int32_t** links = ld == n ? &sp->adj : &sp->adj_ld;
     return dev_alloc(links, sizeof(int32_t) * 18 * (size_t)(ld > 0 ? ld : 1), stream, true);

@@ -503,6 +503,7 @@ struct lbm_state {
                        // then [nblocks * 4] room for the group values of lbm_reduce_flux
   int64_t nblocks;
   bool one_wave;       // at most one_wave_cells(): plain FP32/16-bit steps load links first
+  bool small_list;     // at most small_list_cells()
   unsigned* arrived;   // CTAs of the running flux_sums_kernel that are done
   double* red_host;    // [4] pinned, written by flux_sums_kernel
   int64_t steps;
@@ -518,6 +519,8 @@ namespace lbm {
 // Cells of one wave of the FP32 and 16-bit sweeps on the current device, at
 // their 4 resident 256-thread blocks per SM (0 if the device cannot be asked).
 int64_t one_wave_cells();
+// Lists of more cells take short links and two cells per thread.
+inline int64_t small_list_cells() { return 2 * one_wave_cells(); }
 void free_state(lbm_state* st);
 void free_sparse(lbm_sparse* sp);
 void free_adjoint(lbm_adjoint* ad);

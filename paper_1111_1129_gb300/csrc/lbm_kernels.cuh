@@ -667,8 +667,15 @@ __device__ __forceinline__ uint32_t pack_values(float low, float high) {
 // pulls where they share a word 29,135; link rows through bulk copies into
 // shared memory 36,780; three or four cells per thread 33,154 / 28,450; cells
 // i and i + 32 of a warp's 64 40,189; links loaded before the wait for the
-// previous step 37,263; write-back stores 42,277.  A list whose tiles meet too
-// many pages for short links takes one cell per thread.
+// previous step 37,263; write-back stores 42,277.
+//
+// A large list with a tile that meets too many pages for short links (a thin
+// plate with a slit across the rows does it in lexicographic order) has 32-bit
+// ones.  The 16-bit forms take two cells per thread there too, each link by a
+// load of its own and the cells one after the other: 1024x256x256 box with such
+// a plate, FP16S / BF16S 46,390 / 46,580, one cell 41,670 / 41,710; both cells
+// at once and packed together, as with short links, 45,900 / 46,700.  FP32
+// steps take one cell, 31,830.
 #ifndef LBM_PAIR_THREADS
 #define LBM_PAIR_THREADS 256
 #endif
@@ -692,7 +699,7 @@ __device__ __forceinline__ void load_pair_links(const Links& links, int32_t ld, 
   entry = page_entry(links, i);
 }
 
-template <int PREC, bool DAMPED, bool KEEP_U>
+template <int PREC, bool DAMPED, bool KEEP_U, bool SHORT>
 __global__ void __launch_bounds__(kPairThreads, LBM_PAIR_MIN_BLOCKS)
     sweep_pair_kernel(const typename Form<PREC>::S* __restrict__ src,
                       typename Form<PREC>::S* __restrict__ dst, Links links, int32_t n,
@@ -701,19 +708,29 @@ __global__ void __launch_bounds__(kPairThreads, LBM_PAIR_MIN_BLOCKS)
   static_assert(PREC == LBM_F16S || PREC == LBM_BF16S, "16-bit forms only");
   const int32_t z = prior_step_done();
   const int32_t i = 2 * (int32_t)(blockIdx.x * kPairThreads + threadIdx.x) + z;
-  if (i >= ld) return;   // whole warps: their 64 cells are one tile of links
   const bool two = i + 1 < n;   // false for the last cell of an odd-length list, and past it
   const unsigned short* src16 = reinterpret_cast<const unsigned short*>(src);
-  uint32_t word[18];
-  int32_t entry;
-  load_pair_links(links, ld, i, word, entry);
   int32_t a[18], b[18];
+  if constexpr (SHORT) {
+    if (i >= ld) return;   // whole warps: their 64 cells are one tile of links
+    uint32_t word[18];
+    int32_t entry;
+    load_pair_links(links, ld, i, word, entry);
 #pragma unroll
-  for (int q = 0; q < 18; ++q) {
-    a[q] = short_slot(q + 1, ld, entry, word[q]);
-    b[q] = short_slot(q + 1, ld, entry, word[q] >> 16);
+    for (int q = 0; q < 18; ++q) {
+      a[q] = short_slot(q + 1, ld, entry, word[q]);
+      b[q] = short_slot(q + 1, ld, entry, word[q] >> 16);
+    }
+    if (i >= n) return;
+  } else {
+    if (i >= n) return;
+#pragma unroll
+    for (int q = 0; q < 18; ++q) {
+      const int32_t* p = links.wide + q * ld + i;
+      a[q] = ld_nc(p);
+      b[q] = two ? ld_nc(p + 1) : 0;
+    }
   }
-  if (i >= n) return;
   // pulled values, packed: low half cell i, high half cell i + 1
   uint32_t g[19];
   if (two) {   // the rest row is aligned at even i
@@ -728,21 +745,41 @@ __global__ void __launch_bounds__(kPairThreads, LBM_PAIR_MIN_BLOCKS)
     g[q + 1] = lo | (hi << 16);
   }
   // the arithmetic is that of the stored values, times k.scale
-  float v0[19], v1[19], rho, u0[3], u1[3];
+  uint32_t out[19];
+  float rho, u0[3], u1[3];
+  if constexpr (SHORT) {
+    float v0[19], v1[19];
 #pragma unroll
-  for (int q = 0; q < 19; ++q) {
-    v0[q] = low_value<PREC>(g[q]);
-    v1[q] = high_value<PREC>(g[q]);
+    for (int q = 0; q < 19; ++q) {
+      v0[q] = low_value<PREC>(g[q]);
+      v1[q] = high_value<PREC>(g[q]);
+    }
+    collide<float, DAMPED, true>(v0, k, DAMPED ? ld_nc(alpha + i) : 0.f, rho, u0);
+    if (two) collide<float, DAMPED, true>(v1, k, DAMPED ? ld_nc(alpha + i + 1) : 0.f, rho, u1);
+#pragma unroll
+    for (int q = 0; q < 19; ++q) out[q] = pack_values<PREC>(v0[q], v1[q]);
+  } else {   // one cell after the other, each rounded by itself
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      if (c == 0 || two) {
+        float v[19];
+#pragma unroll
+        for (int q = 0; q < 19; ++q) v[q] = c ? high_value<PREC>(g[q]) : low_value<PREC>(g[q]);
+        collide<float, DAMPED, true>(v, k, DAMPED ? ld_nc(alpha + i + c) : 0.f, rho, c ? u1 : u0);
+#pragma unroll
+        for (int q = 0; q < 19; ++q) {
+          const uint32_t h = pack_values<PREC>(v[q], 0.f);
+          out[q] = c ? out[q] | (h << 16) : h;
+        }
+      }
+    }
   }
-  collide<float, DAMPED, true>(v0, k, DAMPED ? ld_nc(alpha + i) : 0.f, rho, u0);
-  if (two) collide<float, DAMPED, true>(v1, k, DAMPED ? ld_nc(alpha + i + 1) : 0.f, rho, u1);
   unsigned short* dst16 = reinterpret_cast<unsigned short*>(dst);
 #pragma unroll
   for (int q = 0; q < 19; ++q) {
     const int32_t e = q * ld + i;   // even: one 4-byte store of the pair
-    const uint32_t out = pack_values<PREC>(v0[q], v1[q]);
-    if (two) asm volatile("st.global.cs.u32 [%0], %1;" ::"l"(dst16 + e), "r"(out) : "memory");
-    else st_cs(dst16 + e, (unsigned short)(out & 0xffffu));
+    if (two) asm volatile("st.global.cs.u32 [%0], %1;" ::"l"(dst16 + e), "r"(out[q]) : "memory");
+    else st_cs(dst16 + e, (unsigned short)(out[q] & 0xffffu));
   }
   if constexpr (KEEP_U)
 #pragma unroll

@@ -197,9 +197,17 @@ bool valid_state(const lbm_state* st) { return st && st->magic == kMagicState; }
 
 namespace {
 
+template <int PREC, bool DAMPED, bool SHORT>
+auto* pair_kernel(bool keep_u) {
+  return keep_u ? sweep_pair_kernel<PREC, DAMPED, true, SHORT>
+                : sweep_pair_kernel<PREC, DAMPED, false, SHORT>;
+}
+
 // One step of a state from src to dst.  The lists that have short links take
 // two adjacent cells per thread in their plain FP32 and 16-bit steps; a list
-// of one wave loads its links before the wait.
+// of one wave loads its links before the wait.  A list above two waves that
+// has 32-bit links, because one of its tiles meets too many pages, takes two
+// cells per thread in the 16-bit forms alone.
 // u_out: keep the velocity there (a step that does not reduce).
 template <int PREC, bool DAMPED, bool SHORT>
 cudaError_t launch_step(const lbm_state* st, const typename Form<PREC>::S* src,
@@ -219,13 +227,15 @@ cudaError_t launch_step(const lbm_state* st, const typename Form<PREC>::S* src,
                           u_out);
   };
   if (reduce) return sweep(sweep_kernel<PREC, DAMPED, kWarpSums, SHORT>);
-  if constexpr (SHORT && (PREC == LBM_F16S || PREC == LBM_BF16S)) {
-    return u_out ? pair(sweep_pair_kernel<PREC, DAMPED, true>, kPairThreads)
-                 : pair(sweep_pair_kernel<PREC, DAMPED, false>, kPairThreads);
+  constexpr bool k16 = PREC == LBM_F16S || PREC == LBM_BF16S;
+  if constexpr (SHORT && k16) {
+    return pair(pair_kernel<PREC, DAMPED, SHORT>(u_out != nullptr), kPairThreads);
   } else if constexpr (SHORT && (PREC == LBM_F32 || PREC == LBM_F32S)) {
     return u_out ? pair(sweep_pair32_kernel<PREC, DAMPED, true>, kPair32Threads)
                  : pair(sweep_pair32_kernel<PREC, DAMPED, false>, kPair32Threads);
   } else {
+    if constexpr (k16)
+      if (!st->small_list) return pair(pair_kernel<PREC, DAMPED, SHORT>(u_out != nullptr), kPairThreads);
     if constexpr (!SHORT && PREC != LBM_F64)
       if (st->one_wave)
         return u_out ? sweep(sweep_kernel<PREC, DAMPED, kKeepU, false, true>)
@@ -508,6 +518,7 @@ extern "C" int lbm_state_create(const lbm_sparse* sp, int32_t precision, int32_t
   st->nblocks = (n + kSweepThreads - 1) / kSweepThreads;
   if (st->nblocks < 1) st->nblocks = 1;
   st->one_wave = n <= one_wave_cells();
+  st->small_list = n <= small_list_cells();
   // rows of sp->ld elements; the padding slots past n are never read
   const size_t bytes = storage_bytes(precision) * 19 * (size_t)(sp->ld > 0 ? sp->ld : 1);
   const cudaStream_t stream = sp->stream;
