@@ -33,6 +33,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <mutex>
@@ -172,14 +173,25 @@ bool is_shifted(int prec) { return prec == LBM_F32S || prec == LBM_F16S || prec 
 
 static double g_timeout_s = 600.0;
 
+// Waits in progress, in all threads.
+static std::atomic<int> g_waits{0};
+
 int wait_event(cudaEvent_t ev, cudaStream_t stream, double timeout_s) {
   LBM_CUDA_TRY(cudaEventRecord(ev, stream));
   const double limit = timeout_s > 0 ? timeout_s : g_timeout_s;
   // A sleep lasts 70 us or more, as long as a short call; so the first 4 ms
   // are polled without one, and later it is at most 2% of the wait.  (32x32x64
   // bed, one step with its sums and fields: 145 us when every poll slept, 58
-  // us now, with the sums in one launch.)
+  // us now, with the sums in one launch.)  Polls take a core and the driver's
+  // lock, so only the first of many waits do so, one for every four cores: with
+  // 64 threads on 16 cores, 400 steps and their sums each, 13.8 ms a call when
+  // all polled (12 cores busy), 13.2 when none did (3), 13.3 so (3).
   constexpr double kPollS = 4e-3;
+  static const int kPolling = std::max(1, (int)std::thread::hardware_concurrency() / 4);
+  struct Count {
+    const int before = g_waits.fetch_add(1);
+    ~Count() { g_waits.fetch_sub(1); }
+  } count;
   const auto t0 = std::chrono::steady_clock::now();
   for (;;) {
     const cudaError_t e = cudaEventQuery(ev);
@@ -189,7 +201,8 @@ int wait_event(cudaEvent_t ev, cudaStream_t stream, double timeout_s) {
         std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     if (el > limit)
       return fail(LBM_ETIMEOUT, "queued work still running after %.1f s", limit);
-    if (el > kPollS) std::this_thread::sleep_for(std::chrono::microseconds(20));
+    if (el > kPollS || count.before >= kPolling)
+      std::this_thread::sleep_for(std::chrono::microseconds(20));
   }
 }
 
