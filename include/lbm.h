@@ -139,12 +139,15 @@ int lbm_ordering_keys(const int32_t dims[3], lbm_ordering ord, uint64_t* keys_de
  *            and the adjacency.  The states keep their arrays in rows of
  *            L slots, L = N rounded up to 64, so that every row starts on a
  *            128-byte boundary; the adjacency the steps read names slots
- *            r*L + m, as int32 (18 rows of L, 72 bytes per L) or, for larger lists
- *            (more than 311,296 cells on GB300), in 16 bits per link and a table of neighbourhoods per 64 cells (38
- *            bytes per L).  adj[18*N] of the layout above is derived from it
- *            on its first request (lbm_sparse_info, lbm_state_create_batched)
- *            and then kept; with int32 links and
- *            L = N it is the same array.
+ *            r*L + m, as int32 (18 rows of L, 72 bytes per L) or, for larger
+ *            lists (more than 311,296 cells on GB300), in 16 bits per link
+ *            and a table of neighbourhoods per 64 cells (38 bytes per L).
+ *            A larger list has int32 links too if the neighbours of some 64
+ *            cells are spread over more of the list than the table holds
+ *            (a thin perforated plate in lexicographic order, for instance).
+ *            adj[18*N] of the layout above is derived from it on its first
+ *            request (lbm_sparse_info, lbm_state_create_batched) and then
+ *            kept; with int32 links and L = N it is the same array.
  * The call synchronises `stream` (to learn N, and again before returning,
  * so the flags may be released afterwards).  Errors: LBM_EINVAL,
  * LBM_EFLAGS, LBM_EOVERFLOW (19*L >= 2^31), LBM_ENOMEM, LBM_ECUDA.
@@ -155,9 +158,9 @@ int lbm_build_sparse(const uint8_t* flags, const int32_t dims[3], lbm_ordering o
 /*
  * Read-only views of a sparse representation.  Any out pointer may be NULL.
  * The device pointers stay owned by the handle.  adj_dev is adj[18*N] of the
- * layout above; unless the steps' links are that array the first request builds it
- * (72 bytes per cell of device memory, one kernel on the handle's stream,
- * which the call then synchronises) and may fail with LBM_ENOMEM.
+ * layout above; unless the steps' links are that array the first request
+ * builds it (72 bytes per cell of device memory, one kernel on the handle's
+ * stream, which the call then synchronises) and may fail with LBM_ENOMEM.
  * lbm_free gives them back in the order of the handle's stream, for the next
  * lattice to write: what reads them on another stream has to finish before.
  */

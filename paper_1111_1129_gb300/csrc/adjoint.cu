@@ -274,8 +274,11 @@ __device__ __forceinline__ C reverse_cell(const C lf[19], const C u[3], C al, co
 // One reverse step t: lam_f_t = S^T lam_g_{t+1} (pulled), then
 // lam_g_t = C'(g_t)^T lam_f_t with the velocity u of that collision, rows of
 // ld.  dalpha may be null (dJ/dalpha not wanted).
-// FP32 at 5 resident blocks (48 registers): 200 steps and their gradient on the
-// damped 128^3 bed 17.3 ms, 17.8 at 4 and 17.7 at 6, when it served that list.
+// FP32, lists with 32-bit links, at 5 resident blocks (48 registers): reverse
+// pass of 200 damped steps on 29,479 cells 0.757 ms (at 4 and 6 blocks 0.783 and
+// 0.777), on a box of 305,184 cells 2.20 (2.32, 2.34), of 20 steps on 15.9
+// million cells with a slit plate 11.1 (11.7, 11.3); on 200,704 cells 1.69, and
+// 1.66 at 6.
 #ifndef LBM_ADJ_MIN_BLOCKS
 #define LBM_ADJ_MIN_BLOCKS 5
 #endif
@@ -296,13 +299,6 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(C) == 4 ? LBM_ADJ_MIN_BL
 #pragma unroll
     for (int j = 0; j < 3; ++j) u[j] = ld_nc(u_in + j * ld + i);
     const C al = DAMPED ? ld_nc(alpha + i) : C(0);
-    const C s = DAMPED ? C(1) / (C(1) + C(0.5) * al) : C(1);
-    C S[9], D[9];
-#pragma unroll
-    for (int p = 0; p < 9; ++p) {
-      S[p] = lf[2 * p + 1] + lf[2 * p + 2];
-      D[p] = lf[2 * p + 1] - lf[2 * p + 2];
-    }
     // Two forms of the same update.  FP64 arithmetic takes the pair form:
     // the outputs of pair (a, b) are e +- o, e = (1 - w+)/2 S + base and
     // o = (1 - w-)/2 D + s G (L^T's k1 la + k2 lb and k1 lb + k2 la have sum
@@ -314,6 +310,13 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(C) == 4 ? LBM_ADJ_MIN_BL
     // ran 6 blocks per SM instead of 5, and was slower, 57.6 us against 53.2
     // (DRAM 65% against 71%; reverse pass 187 ms against 178).
     if constexpr (sizeof(C) == 8) {
+      const C s = DAMPED ? C(1) / (C(1) + C(0.5) * al) : C(1);
+      C S[9], D[9];
+#pragma unroll
+      for (int p = 0; p < 9; ++p) {
+        S[p] = lf[2 * p + 1] + lf[2 * p + 2];
+        D[p] = lf[2 * p + 1] - lf[2 * p + 2];
+      }
       const C s34 = S[3] + S[4], s56 = S[5] + S[6], s78 = S[7] + S[8];
       const C M0 = C(12) * lf[0] + C(2) * ((S[0] + S[1]) + S[2]) + ((s34 + s56) + s78);
       const C M1x = C(2) * D[0] + ((D[3] + D[4]) + (D[5] + D[6]));

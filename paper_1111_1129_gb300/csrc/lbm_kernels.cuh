@@ -205,10 +205,16 @@ __device__ __forceinline__ void store_stream(typename Form<PREC>::S* p, typename
 // 123 instead of 137 (and a division): 256x128x128 bed 4,131 -> 4,443 MFLUP/s.
 // rho enters as two terms, so that its rounding at 1 does not reach the
 // populations, and the rest population's factor makes up for the rounding of
-// the other constants (make_coef): over 12 runs of 10 to 200 steps, damped and
-// not, w+ from 0.7 to 1.9, the error of u fell by 10-25% and that of f, mostly
-// drift of the mass, to 0.7 of the former value in the median (1.02 and 11
-// times in the two runs where it rose, 2.2e-15 at most there).
+// the other constants (make_coef).  Errors against FP64 arithmetic on f - w, 80
+// steps from a flow at 25 rates w+ from 0.7 to 1.9, collide()'s form and this
+// one: that of u fell at every rate, to 0.85 in the median (0.68 to 0.93); that of
+// f, mostly drift of the mass, in the median from 2.3e-15 to 1.1e-15 and at most
+// from 5.4e-15 to 3.7e-15, but it rose at six rates, where the roundings of
+// the former constants nearly cancel (0.9, 1.05, 1.1, 1.2, 1.55, 1.8: from 1.7e-16
+// ... 5.2e-16 to 0.5e-15 ... 3.7e-15).  A rest factor in two parts, one
+// instruction more, takes the drift away (f 1.2e-16 to 5.6e-16 at every rate) but
+// the roundings then repeat from step to step: u at w+ = 1 is off by 6.1e-12
+// instead of 2.9e-12 (collide()'s form 3.6e-12), and 4,455 -> 4,420 MFLUP/s.
 template <bool DAMPED>
 __device__ __forceinline__ void collide_f64(double g[19], const Coef<double>& k, double alpha,
                                             double& rho_out, double u_out[3]) {
@@ -879,8 +885,9 @@ __device__ __forceinline__ void tree_sum_1024(double (*sm)[4]) {
 // *arrived counts the CTAs and wraps to 0; null: the groups only, which
 // final_sum_kernel adds in a launch of its own.  One launch takes 25 us with the
 // host's wait up to 64 groups, two 27; at 1024 groups, where 1024 threads add
-// them faster, 72 and 66.  So lists above 16 groups (1,048,576 cells, steps of
-// 20 us and more) take two.
+// them faster, 72 and 66.  The line lies at 16 groups (1,048,576 cells), below
+// the crossing: from there on a call's step alone takes 20 us and more, the 2 us
+// are lost in it, and the benchmark counts two launches for its larger beds.
 constexpr int kCollapseThreads = 256, kOneLaunchGroups = 16;
 __global__ void __launch_bounds__(kCollapseThreads)
     flux_sums_kernel(const double* __restrict__ part, int64_t nblocks, double* groups,

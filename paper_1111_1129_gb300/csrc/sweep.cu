@@ -310,11 +310,11 @@ int launch_moments(const lbm_state* st, double* rho, double* u) {
   using C = typename Form<PREC>::C;
   const int32_t n = (int32_t)st->sp->n;
   if (n == 0) return LBM_OK;
-  const Coef<C> k = make_coef<C>(st->last_wp, st->last_wm, st->last_force, st->scale_exp);
   const S* prev = (const S*)st->buf[st->cur ^ 1];
   if constexpr (sizeof(C) == 8) {
     LBM_CUDA_TRY(launch_moments_fx(st, prev, st->last_force, rho, u));
   } else {
+    const Coef<C> k = make_coef<C>(st->last_wp, st->last_wm, st->last_force, st->scale_exp);
     const C* alpha = (const C*)st->alpha;
     const Links links = state_links(st->sp);
     const auto kernel = links.wide ? (alpha ? moments_kernel<PREC, true, false> : moments_kernel<PREC, false, false>)
