@@ -118,12 +118,12 @@ class SparseLattice:
         self.ordering = ordering
         self.block = tuple(block)
         self.periodic = int(periodic)
-        self._reads = {}   # the last copy queued on each stream but the lattice's own
+        self._own_stream = int(self.stream.cuda_stream)
+        self._reads = []   # copies queued on other streams, not known to have finished
         self._handle = None
         self._handle = capi.lbm_build_sparse(
             flags.data_ptr(), self.dims,
-            capi.make_ordering(ORDERINGS[ordering], block, periodic),
-            int(self.stream.cuda_stream))
+            capi.make_ordering(ORDERINGS[ordering], block, periodic), self._own_stream)
         # the public links are built on first request (adjacency())
         self.n, self._cells, _, self._inv = capi.lbm_sparse_info(self._handle, want_adj=False)
         self._adj = 0
@@ -135,13 +135,15 @@ class SparseLattice:
     def _copy(self, ptr: int, shape) -> torch.Tensor:
         """Copy of int32 device memory of the handle, on the current stream.
         The handle gives its memory back in the order of the lattice's own
-        stream, for the next lattice to write; so close() waits for the last
-        copy queued on any other."""
+        stream, for the next lattice to write; so close() waits for copies
+        queued on any other."""
         out = _borrow(ptr, shape, "<i4", torch.int32).clone()
-        here = torch.cuda.current_stream()
-        if (here.cuda_stream != self.stream.cuda_stream
-                and not torch.cuda.is_current_stream_capturing()):
-            self._reads[here.cuda_stream] = here.record_event()
+        # the handle alone: a Stream object for every copy cost 28 us in a
+        # request for all three arrays, which takes 80 for a small bed
+        here = torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        if here != self._own_stream and not torch.cuda.is_current_stream_capturing():
+            queued = [copied for copied in self._reads if not copied.query()]
+            self._reads = queued + [torch.cuda.current_stream().record_event()]
         return out
 
     def cells(self) -> torch.Tensor:
@@ -168,7 +170,7 @@ class SparseLattice:
         if self._handle:
             handle, self._handle = self._handle, None
             try:
-                for copied in self._reads.values():
+                for copied in self._reads:
                     copied.synchronize()
             finally:
                 capi.lbm_free(handle)
